@@ -823,7 +823,16 @@ int gw_model_create(gw_ctx_t ctx, const gw_model_desc* d, gw_model_t* out) {
     p += layer_param_count(s);
     LayerDev L;
     L.s = s;
-    std::vector<float> w32(wf.begin(), wf.end()), b32(bf.begin(), bf.end());
+    std::vector<float> w32(conv_f32_weight_floats(s.cin, s.cout, s.k), 0.f), b32(bf.begin(), bf.end());
+    {
+      // [C_out][C_in K] -> [C_in K][C_out padded], in blocks that stay in cache
+      const int rows = s.cout, cols = s.cin * s.k, cop = conv_f32_cop(s.cout);
+      for (int r0 = 0; r0 < rows; r0 += 16)
+        for (int c0 = 0; c0 < cols; c0 += 16)
+          for (int c = c0; c < std::min(c0 + 16, cols); ++c)
+            for (int r = r0; r < std::min(r0 + 16, rows); ++r)
+              w32[(size_t)c * cop + r] = (float)wf[(size_t)r * cols + c];
+    }
     wfold.push_back(wf);
     bfold.push_back(b32);
     L.w = upload(m, w32);

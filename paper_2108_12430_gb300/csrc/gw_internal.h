@@ -68,7 +68,7 @@ std::vector<LayerSpec> bbhnet_specs(int n_in);
 // Weights of one layer on the device after the BatchNorm fold.
 struct LayerDev {
   LayerSpec s;
-  float* w = nullptr;      // FP32 [C_out][C_in][K] (transposed convs re-indexed to this order)
+  float* w = nullptr;      // FP32 weights [C_in][K][conv_f32_cop(C_out)]
   float* b = nullptr;      // FP32 [C_out]
   // tensor-core path (BF16 / FP8): packed operand image and per-K-step table
   void* wq = nullptr;      // packed B operand image (bf16 or e4m3)
@@ -198,12 +198,17 @@ int current_sm_count();
 void* dev_alloc(gw_ctx* ctx, size_t bytes, size_t* counter);
 void dev_free(gw_ctx* ctx, void* p, size_t bytes, size_t* counter);
 
-// ---- FP32 SIMT kernels (k_f32.cu) --------------------------------------------
+// ---- FP32 SIMT kernels (k_conv_f32.cu, k_f32.cu) -----------------------------
+// Weights of the FP32 conv kernel: [C_in][K][cop], output channels innermost
+// and zero-padded to a multiple of 8, so that a CTA's channels of one tap are
+// one contiguous, 16-byte aligned row.
+__host__ __device__ inline int conv_f32_cop(int cout) { return (cout + 7) / 8 * 8; }
+inline size_t conv_f32_weight_floats(int cin, int cout, int k) { return (size_t)cin * k * conv_f32_cop(cout); }
 struct ConvF32Args {
   const float* x; int64_t xb, xc;     // input element (b, c, t) at x + b*xb + c*xc + t
   float* y; int64_t yb, yc;           // output element (b, c, t)
   const float* res; int64_t rb, rc;   // optional residual added before the activation
-  const float* w; const float* bias;  // folded weights [C_out][C_in][K], bias [C_out]
+  const float* w; const float* bias;  // folded weights [C_in][K][conv_f32_cop(C_out)], bias [C_out]
   const float* in_mean; const float* in_istd;  // optional input standardisation
   const float* const* item_ptr;       // optional device table: address of item b's (0, 0) (replaces x + b*xb)
   const float* gy; int64_t gyb, gyc;  // optional: multiply the output by act'(gy) (gy = that activation's output)

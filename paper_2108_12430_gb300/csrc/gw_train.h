@@ -15,8 +15,8 @@ struct FoldArgs {
   const float* p;             // raw parameters (device)
   int64_t off_w, off_b, off_g, off_be, off_mu, off_var;
   int cin, cout, K, transposed, bn;
-  float* wf;                  // folded [C_out][C_in][K]
-  float* wT;                  // folded, transposed [C_in][C_out][K]
+  float* wf;                  // folded [C_in][K][conv_f32_cop(C_out)]
+  float* wT;                  // folded, transposed [C_out][K][conv_f32_cop(C_in)]
   float* bf;                  // folded bias [C_out]
 };
 

@@ -28,9 +28,10 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
   return t;  // valid in thread 0
 }
 
-// Folded weights of one layer in the device layout [C_out][C_in][K] (wf),
-// the same values transposed to [C_in][C_out][K] (wT, the data-gradient
-// kernel's weights) and the folded bias (bf):
+// Folded weights of one layer in the conv kernel's layout [C_in][K][C_out
+// padded] (wf), the same values with the channels exchanged, [C_out][K][C_in
+// padded] (wT, the data gradient's weights), and the folded bias (bf); the
+// padding is zero from the start and never written:
 //   sc[o] = gamma[o] / sqrt(var[o] + eps),  w' = w sc[o],  b' = (b - mean) sc + beta.
 __device__ __forceinline__ void fold_body(const FoldArgs& f) {
   const int n = f.cout * f.cin * f.K;
@@ -40,8 +41,8 @@ __device__ __forceinline__ void fold_body(const FoldArgs& f) {
     double sc = 1.0;
     if (f.bn) sc = (double)f.p[f.off_g + o] / sqrt((double)f.p[f.off_var + o] + (double)kBnEps);
     const float w = (float)((double)f.p[f.off_w + raw] * sc);
-    f.wf[e] = w;
-    f.wT[((int64_t)i * f.cout + o) * f.K + k] = w;
+    f.wf[((int64_t)i * f.K + k) * conv_f32_cop(f.cout) + o] = w;
+    f.wT[((int64_t)o * f.K + k) * conv_f32_cop(f.cin) + i] = w;
   }
   for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < f.cout; o += gridDim.x * blockDim.x) {
     const double b = f.p[f.off_b + o];

@@ -255,9 +255,8 @@ int gw_trainer_create(gw_ctx_t ctx, const gw_trainer_desc* d, const float* in_me
     t->n_params = (size_t)off;
     const int Bm = d->max_batch;
     for (auto& T : t->layers) {
-      const size_t nw = (size_t)T.s.cin * T.s.cout * T.s.k;
-      T.f.wf = talloc<float>(t, nw);
-      T.f.wT = talloc<float>(t, nw);
+      T.f.wf = talloc<float>(t, conv_f32_weight_floats(T.s.cin, T.s.cout, T.s.k));
+      T.f.wT = talloc<float>(t, conv_f32_weight_floats(T.s.cout, T.s.cin, T.s.k));
       T.f.bf = talloc<float>(t, T.s.cout);
     }
     std::vector<float> mean(d->n_in, 0.f), istd(d->n_in, 1.f);
@@ -290,7 +289,7 @@ int gw_trainer_create(gw_ctx_t ctx, const gw_trainer_desc* d, const float* in_me
     t->zero_bias = talloc<float>(t, max_c);
     t->err = talloc<int>(t, 1);
     if (t->tc_data) {
-      // per layer: the forward conv (weights: wf, as stored) and the conv that
+      // per layer: the forward conv (weights: wf) and the conv that
       // maps its output gradient to its input gradient (weights: wT; a
       // stride-2 conv's is a transposed conv and vice versa, a stride-1 conv's
       // is a stride-1 conv with the taps reversed and padding K - 1 - p)
@@ -300,7 +299,10 @@ int gw_trainer_create(gw_ctx_t ctx, const gw_trainer_desc* d, const float* in_me
         const LayerSpec& s = T.s;
         const size_t nw = (size_t)s.cin * s.cout * s.k;
         std::vector<int32_t> src(nw);
-        for (size_t i = 0; i < nw; ++i) src[i] = (int32_t)i;
+        for (int o = 0; o < s.cout; ++o)
+          for (int c = 0; c < s.cin; ++c)
+            for (int k = 0; k < s.k; ++k)
+              src[((size_t)o * s.cin + c) * s.k + k] = (c * s.k + k) * conv_f32_cop(s.cout) + o;
         T.tf.s = s;
         T.tf.b = T.f.bf;
         tc_prepare_trainable(T.tf, ctx, &t->tc_bytes, t->tc_allocs, src, &T.map_f, &T.n_f);
@@ -323,11 +325,13 @@ int gw_trainer_create(gw_ctx_t ctx, const gw_trainer_desc* d, const float* in_me
           ds.transposed = false;
           ds.stride = 1;
           ds.pad_l = ds.pad_r = s.k - 1 - s.pad_l;
-          for (int c = 0; c < s.cin; ++c)
-            for (int o = 0; o < s.cout; ++o)
-              for (int k = 0; k < s.k; ++k)
-                src[((size_t)c * s.cout + o) * s.k + k] = (int32_t)(((size_t)c * s.cout + o) * s.k + (s.k - 1 - k));
         }
+        for (int c = 0; c < s.cin; ++c)
+          for (int o = 0; o < s.cout; ++o)
+            for (int k = 0; k < s.k; ++k) {
+              const int kk = s.stride == 2 ? k : s.k - 1 - k;
+              src[((size_t)c * s.cout + o) * s.k + k] = (o * s.k + kk) * conv_f32_cop(s.cin) + c;
+            }
         T.td.s = ds;
         T.td.b = t->zero_bias;
         tc_prepare_trainable(T.td, ctx, &t->tc_bytes, t->tc_allocs, src, &T.map_d, &T.n_d);
