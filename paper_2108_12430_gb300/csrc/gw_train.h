@@ -20,17 +20,16 @@ struct FoldArgs {
   float* bf;                  // folded bias [C_out]
 };
 
-// Weight-gradient GEMM: P[chunk][a][c][k] = sum_t A[b][a][t] Bv(b, c, s t + k - p).
+// Weight-gradient contraction dW[a][c][k] = sum_{b,t} A[b][a][t] Bv(b, c, s t + k - p)
+// (Bv = Bm inside [0, LB), 0 outside) and the bias gradient: 1 = sum_t
+// A[a][t] (conv: A is the output gradient), 2 = sum_u Bm[c][u] (transposed
+// conv: Bm is the output gradient; needs LB = s LA and p + s <= K), 0 = none.
 struct WgradArgs {
   const float* A; int64_t ab, aa; int NA, LA;
   const float* Bm; int64_t bb, bc; int NC, LB;
   int K, s, p;
-  int AB, T, chunks_per_b, nj;
+  int bias;
   float* partial;
-  // tensor-core kernel only: also the bias gradient, 1 = sum_t A[a][t] (conv:
-  // A is the output gradient), 2 = sum_u Bm[c][u] (transposed conv: Bm is the
-  // output gradient; needs LB = s LA and p + s <= K)
-  int bias = 0;
 };
 
 void launch_fold(const FoldArgs& f, cudaStream_t st);
@@ -48,11 +47,19 @@ struct UnfoldItem {
   const float* dbf;
 };
 void launch_unfold_many(const UnfoldItem* u, int n, float* dp, cudaStream_t st);
-WgradArgs plan_wgrad(int NA, int NC, int K, int s, int LA);
-size_t wgrad_smem(const WgradArgs& w);
-// w.partial must hold B * w.chunks_per_b * NA * NC * K floats; out gets NA * NC * K.
-void launch_wgrad_partial(const WgradArgs& w, int B, cudaStream_t st);
-void launch_wgrad_reduce(const WgradArgs& w, int B, float* out, cudaStream_t st);
+// FP32 (k_wgrad_f32.cu).  launch_wgrad_f32 writes per-CTA partials
+// (w.partial: wgrad_f32_partial_floats) and returns what launch_wgrad_reduce
+// needs to add them into out (NA * NC * K floats) and db; several layers go
+// into one reduction.
+struct WgradReduceItem {
+  const float* partial;
+  int parts, cols, n_w;  // partials of `cols` floats: n_w weights, then the bias
+  float *out, *db;
+};
+constexpr int kWgradReduceMax = 16;
+size_t wgrad_f32_partial_floats(const WgradArgs& w, int B);
+WgradReduceItem launch_wgrad_f32(const WgradArgs& w, int B, float* out, float* db, cudaStream_t st);
+void launch_wgrad_reduce(const WgradReduceItem* items, int n, cudaStream_t st);
 // The same weight gradient on the tensor cores (BF16 operands, FP32
 // accumulation; k_wgrad_tc.cu): out gets NA * NC * K floats and, with
 // w.bias, db the bias gradient (NA floats for bias 1, NC for bias 2); partial
@@ -60,9 +67,6 @@ void launch_wgrad_reduce(const WgradArgs& w, int B, float* out, cudaStream_t st)
 bool wgrad_tc_supported(const WgradArgs& w);
 size_t wgrad_tc_partial_floats(const WgradArgs& w, int B);
 void launch_wgrad_tc(const WgradArgs& w, int B, float* partial, float* out, float* db, int* err, cudaStream_t st);
-// out[n] = sum_{b, t} G[b][n][t]; part holds B * N floats.
-void launch_bias_grad(const float* G, int64_t gb, int64_t gn, int B, int N, int L, float* part, float* out,
-                      cudaStream_t st);
 void launch_standardise(const float* x, int B, int C, int L, const float* mean, const float* istd, float* y,
                         cudaStream_t st);
 // loss = (1 / (B Lr)) sum r^2 with r = g (*) (strain - y_hat) valid (Lr = L - K + 1);

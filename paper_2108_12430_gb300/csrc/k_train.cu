@@ -1,11 +1,10 @@
-// Training kernels (FP32): BatchNorm fold and its chain rule, weight and bias
-// gradients of conv / transposed-conv layers, the band-limited loss and Adam.
+// Training kernels (FP32): BatchNorm fold and its chain rule, the band-limited
+// loss and Adam (weight gradients: k_wgrad_f32.cu, k_wgrad_tc.cu).
 //
 // Data gradients reuse the forward conv kernel (a conv's data gradient is a
 // transposed conv with the transposed weights and vice versa), with the
 // activation derivative fused into its epilogue.  Every reduction here runs
-// in a fixed order (per-chunk partials, then a sum over chunks), so a
-// gradient is bitwise reproducible.
+// in a fixed order, so a gradient is bitwise reproducible.
 #include "gw_train.h"
 
 namespace gw {
@@ -13,7 +12,6 @@ namespace gw {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kMaxJ = 32;  // weight-gradient outputs per thread
 
 __device__ __forceinline__ float block_sum(float v, float* red) {
 #pragma unroll
@@ -107,85 +105,6 @@ __global__ void unfold_many_kernel(const __grid_constant__ UnfoldList l, float* 
   const UnfoldItem& u = l.u[blockIdx.y];
   if ((int)blockIdx.x >= u.f.cout) return;
   unfold_body(u.f, u.dWf, u.dw_in_major, u.dbf, dp, blockIdx.x);
-}
-
-// Weight-gradient partials of one chunk of (item, positions):
-//   P[chunk][a][c][k] = sum_{t in chunk} A[b][a][t] Bv(b, c, s t + k - p),
-// Bv = Bm inside [0, LB), 0 outside.  Conv: A = output gradient, Bm = input;
-// transposed conv: A = input, Bm = output gradient.  CTA: AB values of a (a
-// power of two), all (c, k), T positions; the A tile (rows padded by one
-// float against bank conflicts) and the B span sit in shared memory.  Thread:
-// one a (AB groups of 256 / AB threads) and NJ of the (c, k) outputs, so one
-// A value feeds NJ multiply-adds per position.  NJ is a compile-time bound
-// (>= w.nj) so that the inner loop has no idle slots.
-template <int NJ>
-__global__ void __launch_bounds__(kThreads) wgrad_partial_kernel(WgradArgs w) {
-  extern __shared__ float sm[];
-  const int chunk = blockIdx.x, b = chunk / w.chunks_per_b, t0 = (chunk % w.chunks_per_b) * w.T;
-  const int a0 = blockIdx.y * w.AB;
-  const int span = w.s * (w.T - 1) + w.K;
-  const int as = w.T + 1;
-  float* As = sm;                 // [AB][T + 1]
-  float* Bs = sm + w.AB * as;     // [NC][span]
-  const int q0 = w.s * t0 - w.p;
-  for (int e = threadIdx.x; e < w.AB * w.T; e += blockDim.x) {
-    const int al = e / w.T, t = e % w.T;
-    const int a = a0 + al, tt = t0 + t;
-    As[al * as + t] = (a < w.NA && tt < w.LA) ? w.A[(int64_t)b * w.ab + (int64_t)a * w.aa + tt] : 0.f;
-  }
-  for (int e = threadIdx.x; e < w.NC * span; e += blockDim.x) {
-    const int c = e / span, q = q0 + e % span;
-    Bs[e] = (q >= 0 && q < w.LB) ? w.Bm[(int64_t)b * w.bb + (int64_t)c * w.bc + q] : 0.f;
-  }
-  __syncthreads();
-  const int tpa = kThreads / w.AB;          // threads per a
-  const int al = threadIdx.x / tpa, ck0 = threadIdx.x % tpa;
-  const int nck = w.NC * w.K;
-  float acc[NJ];
-  int boff[NJ];
-#pragma unroll
-  for (int j = 0; j < NJ; ++j) {
-    acc[j] = 0.f;
-    const int ck = ck0 + j * tpa;
-    boff[j] = ck < nck ? (ck / w.K) * span + ck % w.K : 0;
-  }
-  const float* arow = As + al * as;
-  const int tmax = min(w.T, w.LA - t0);
-  const int s = w.s;
-  for (int t = 0; t < tmax; ++t) {
-    const float av = arow[t];
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) acc[j] = fmaf(av, Bs[boff[j] + s * t], acc[j]);
-  }
-  if (a0 + al < w.NA) {
-    float* out = w.partial + (int64_t)chunk * w.NA * nck + (int64_t)(a0 + al) * nck;
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      const int ck = ck0 + j * tpa;
-      if (ck < nck) out[ck] = acc[j];
-    }
-  }
-}
-
-// out[e] = sum_{ch < n_chunks} P[ch][e] in chunk order.
-__global__ void reduce_chunks_kernel(const float* __restrict__ P, int64_t n, int n_chunks, float* __restrict__ out) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int c = 0; c < n_chunks; ++c) s += P[(int64_t)c * n + e];
-    out[e] = s;
-  }
-}
-
-// part[b][n] = sum_t G[b][n][t] (one CTA per (n, b)).
-__global__ void rowsum_kernel(const float* __restrict__ G, int64_t gb, int64_t gn, int L, int N,
-                              float* __restrict__ part) {
-  __shared__ float red[kThreads / 32];
-  const int n = blockIdx.x, b = blockIdx.y;
-  const float* row = G + (int64_t)b * gb + (int64_t)n * gn;
-  float s = 0.f;
-  for (int t = threadIdx.x; t < L; t += blockDim.x) s += row[t];
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) part[(int64_t)b * N + n] = s;
 }
 
 // x_std[b][c][t] = (x[b][c][t] - mean[c]) / std[c]
@@ -297,72 +216,6 @@ void launch_unfold_many(const UnfoldItem* u, int n, float* dp, cudaStream_t st) 
     mx = std::max(mx, u[i].f.cout);
   }
   unfold_many_kernel<<<dim3(mx, n), kThreads, 0, st>>>(l, dp);
-  GW_LAUNCH_CHECK();
-}
-
-WgradArgs plan_wgrad(int NA, int NC, int K, int s, int LA) {
-  WgradArgs w{};
-  w.NA = NA;
-  w.NC = NC;
-  w.K = K;
-  w.s = s;
-  w.LA = LA;
-  // AB: the largest power of two <= min(16, NA) whose thread groups still
-  // cover the (c, k) outputs with at most kMaxJ per thread
-  w.AB = 1;
-  while (w.AB * 2 <= std::min(16, NA) && (NC * K + kThreads / (w.AB * 2) - 1) / (kThreads / (w.AB * 2)) <= kMaxJ)
-    w.AB *= 2;
-  w.T = 256;
-  while (w.T > 32 && wgrad_smem(w) > 160 * 1024) w.T /= 2;
-  w.chunks_per_b = (LA + w.T - 1) / w.T;
-  const int tpa = kThreads / w.AB;
-  w.nj = (NC * K + tpa - 1) / tpa;
-  return w;
-}
-
-size_t wgrad_smem(const WgradArgs& w) {
-  return ((size_t)w.AB * (w.T + 1) + (size_t)w.NC * (w.s * (w.T - 1) + w.K)) * sizeof(float);
-}
-
-void launch_wgrad_partial(const WgradArgs& w, int B, cudaStream_t st) {
-  GW_CHECK_ARG(w.nj <= kMaxJ, "weight gradient tile too large");
-  const size_t smem = wgrad_smem(w);
-  GW_CHECK_ARG(smem <= 200 * 1024, "weight gradient tile exceeds shared memory");
-  set_smem_limit_once(wgrad_partial_kernel<1>, 200 * 1024);
-  set_smem_limit_once(wgrad_partial_kernel<2>, 200 * 1024);
-  set_smem_limit_once(wgrad_partial_kernel<4>, 200 * 1024);
-  set_smem_limit_once(wgrad_partial_kernel<8>, 200 * 1024);
-  set_smem_limit_once(wgrad_partial_kernel<16>, 200 * 1024);
-  set_smem_limit_once(wgrad_partial_kernel<32>, 200 * 1024);
-  const int n_chunks = B * w.chunks_per_b;
-  dim3 grid(n_chunks, (w.NA + w.AB - 1) / w.AB);
-  if (w.nj <= 1)
-    wgrad_partial_kernel<1><<<grid, kThreads, smem, st>>>(w);
-  else if (w.nj <= 2)
-    wgrad_partial_kernel<2><<<grid, kThreads, smem, st>>>(w);
-  else if (w.nj <= 4)
-    wgrad_partial_kernel<4><<<grid, kThreads, smem, st>>>(w);
-  else if (w.nj <= 8)
-    wgrad_partial_kernel<8><<<grid, kThreads, smem, st>>>(w);
-  else if (w.nj <= 16)
-    wgrad_partial_kernel<16><<<grid, kThreads, smem, st>>>(w);
-  else
-    wgrad_partial_kernel<32><<<grid, kThreads, smem, st>>>(w);
-  GW_LAUNCH_CHECK();
-}
-
-void launch_wgrad_reduce(const WgradArgs& w, int B, float* out, cudaStream_t st) {
-  const int n_chunks = B * w.chunks_per_b;
-  const int64_t n = (int64_t)w.NA * w.NC * w.K;
-  reduce_chunks_kernel<<<grid_for(n), kThreads, 0, st>>>(w.partial, n, n_chunks, out);
-  GW_LAUNCH_CHECK();
-}
-
-void launch_bias_grad(const float* G, int64_t gb, int64_t gn, int B, int N, int L, float* part, float* out,
-                      cudaStream_t st) {
-  rowsum_kernel<<<dim3(N, B), kThreads, 0, st>>>(G, gb, gn, L, N, part);
-  GW_LAUNCH_CHECK();
-  reduce_chunks_kernel<<<grid_for(N), kThreads, 0, st>>>(part, N, B, out);
   GW_LAUNCH_CHECK();
 }
 

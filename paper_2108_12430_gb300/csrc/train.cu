@@ -43,16 +43,19 @@ struct TrainLayer {
 
 // The weight-gradient contraction of a layer (operand pointers left to the
 // caller): conv, A = the output gradient and Bm = the input; transposed conv,
-// A = the input and Bm = the output gradient.  The tensor-core kernel also
-// gives the bias gradient (bias 1: conv, 2: transposed conv).
+// A = the input and Bm = the output gradient; the bias gradient comes with it
+// (bias 1: conv, 2: transposed conv).
 WgradArgs wgrad_plan(const TrainLayer& T) {
   const LayerSpec& s = T.s;
-  WgradArgs w = s.transposed ? plan_wgrad(s.cin, s.cout, s.k, s.stride, T.lin)
-                             : plan_wgrad(s.cout, s.cin, s.k, s.stride, T.lout);
+  WgradArgs w{};
+  w.NA = s.transposed ? s.cin : s.cout;
+  w.NC = s.transposed ? s.cout : s.cin;
+  w.LA = s.transposed ? T.lin : T.lout;
   w.LB = s.transposed ? T.lout : T.lin;
+  w.K = s.k;
+  w.s = s.stride;
   w.p = s.pad_l;
   w.bias = s.transposed ? 2 : 1;
-  if (!wgrad_tc_supported(w)) w.bias = 0;
   return w;
 }
 
@@ -77,10 +80,9 @@ struct gw_trainer {
   std::vector<float*> act;  // output of layer l (l < n_layers - 1), or null when recomputed
   float* scratch = nullptr; // recomputed activation
   float* dv[2] = {nullptr, nullptr};
-  float* partial = nullptr;
+  std::vector<float*> partial;  // per layer: the weight gradient's per-CTA partials
   // per layer: the folded parameters' gradients, unfolded after the backward
   std::vector<float*> dWf, dbf;
-  float* bpart = nullptr;
   float* zero_bias = nullptr;
   const float* params = nullptr;  // raw parameters of the last forward
   int B = 0;
@@ -217,7 +219,8 @@ int gw_trainer_create(gw_ctx_t ctx, const gw_trainer_desc* d, const float* in_me
     const auto specs = deepclean_specs(d->n_in);
     int64_t off = 0;
     int lin = d->length;
-    size_t max_act = 0, max_partial = 0;
+    size_t max_act = 0;
+    std::vector<size_t> n_partial;
     int max_c = 0;
     for (const auto& s : specs) {
       TrainLayer T;
@@ -242,12 +245,10 @@ int gw_trainer_create(gw_ctx_t ctx, const gw_trainer_desc* d, const float* in_me
         off += 4 * s.cout;
       }
       max_act = std::max(max_act, (size_t)std::max(s.cin * T.lin, s.cout * T.lout));
-      const size_t nw = (size_t)s.cin * s.cout * s.k;
       max_c = std::max(max_c, std::max(s.cin, s.cout));
       const WgradArgs w = wgrad_plan(T);
-      max_partial = std::max(max_partial, (size_t)d->max_batch * w.chunks_per_b * nw);
-      if (d->precision == GW_BF16 && wgrad_tc_supported(w))
-        max_partial = std::max(max_partial, wgrad_tc_partial_floats(w, d->max_batch));
+      n_partial.push_back(d->precision == GW_BF16 && wgrad_tc_supported(w) ? wgrad_tc_partial_floats(w, d->max_batch)
+                                                                           : wgrad_f32_partial_floats(w, d->max_batch));
       t->layers.push_back(T);
       lin = T.lout;
     }
@@ -280,12 +281,11 @@ int gw_trainer_create(gw_ctx_t ctx, const gw_trainer_desc* d, const float* in_me
     if (t->checkpoint) t->scratch = talloc<float>(t, (size_t)Bm * max_act);
     t->dv[0] = talloc<float>(t, (size_t)Bm * max_act);
     t->dv[1] = talloc<float>(t, (size_t)Bm * max_act);
-    t->partial = talloc<float>(t, max_partial);
+    for (size_t n : n_partial) t->partial.push_back(talloc<float>(t, n));
     for (const TrainLayer& T : t->layers) {
       t->dWf.push_back(talloc<float>(t, (size_t)T.s.cin * T.s.cout * T.s.k));
       t->dbf.push_back(talloc<float>(t, T.s.cout));
     }
-    t->bpart = talloc<float>(t, (size_t)Bm * max_c);
     t->zero_bias = talloc<float>(t, max_c);
     t->err = talloc<int>(t, 1);
     if (t->tc_data) {
@@ -444,6 +444,7 @@ int gw_trainer_backward(gw_trainer_t t, const float* dy_hat, float* dparams, voi
   const float* g = dy_hat;  // gradient w.r.t. the current layer's (pre-activation) output
   int64_t gb = t->L, gn = t->L;
   int cur = 0;
+  std::vector<WgradReduceItem> reduce;  // FP32 weight gradients: added up by one launch at the end
   TcOut gnext{};  // tc_data: the next data gradient's input, blocked by the previous one
   for (int l = nl - 1; l >= 0; --l) {
     const TrainLayer& T = t->layers[l];
@@ -463,27 +464,13 @@ int gw_trainer_backward(gw_trainer_t t, const float* dy_hat, float* dparams, voi
       w.A = xin; w.ab = xb; w.aa = xc;
       w.Bm = g; w.bb = gb; w.bc = gn;
     }
-    w.partial = t->partial;
-    bool db_done = false;
+    w.partial = t->partial[l];
     if (t->wgrad_tc && wgrad_tc_supported(w)) {
-      // the bias gradient comes with the weight gradient (a row of ones in the GEMM)
       Prof p(l < 8 ? kWgradTcNames[l] : "train.wgrad_tc", st);
-      launch_wgrad_tc(w, B, t->partial, t->dWf[l], w.bias ? t->dbf[l] : nullptr, t->err, st);
-      db_done = w.bias != 0;
+      launch_wgrad_tc(w, B, w.partial, t->dWf[l], t->dbf[l], t->err, st);
     } else {
-      w.bias = 0;
-      {
-        Prof p(l < 8 ? kWgradNames[l] : "train.wgrad", st);
-        launch_wgrad_partial(w, B, st);
-      }
-      {
-        Prof p("train.wgrad_reduce", st);
-        launch_wgrad_reduce(w, B, t->dWf[l], st);
-      }
-    }
-    if (!db_done) {
-      Prof p("train.bgrad", st);
-      launch_bias_grad(g, gb, gn, B, s.cout, T.lout, t->bpart, t->dbf[l], st);
+      Prof p(l < 8 ? kWgradNames[l] : "train.wgrad", st);
+      reduce.push_back(launch_wgrad_f32(w, B, t->dWf[l], t->dbf[l], st));
     }
     if (l == 0) break;
     // data gradient, times the derivative of layer l-1's activation (whose
@@ -564,6 +551,10 @@ int gw_trainer_backward(gw_trainer_t t, const float* dy_hat, float* dparams, voi
     gb = xb;
     gn = xc;
     cur ^= 1;
+  }
+  for (size_t i = 0; i < reduce.size(); i += kWgradReduceMax) {
+    Prof p("train.wgrad_reduce", st);
+    launch_wgrad_reduce(reduce.data() + i, (int)std::min<size_t>(kWgradReduceMax, reduce.size() - i), st);
   }
   {
     // every layer's chain rule from the folded to the raw parameters, one launch
