@@ -1175,7 +1175,7 @@ int gw_whiten(gw_fir_t f, const float* x, int B, int C, int L_in, float* y, void
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (f->precision == GW_FP32) {
     Prof p("fir_f32", st);
-    launch_fir_f32(x, L_in, y, lout, B * C, f->d_taps, f->ntaps, lout, st);
+    launch_fir_f32(fir_valid_args(x, L_in, y, lout, f->d_taps, f->ntaps, lout), B * C, st);
   } else {
     GW_CHECK_ARG(L_in % 8 == 0, "BF16 whitening needs L_in a multiple of 8");
     const int lin8 = L_in / 8, lout8 = lout / 8;

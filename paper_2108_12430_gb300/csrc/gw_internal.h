@@ -218,10 +218,30 @@ struct ConvF32Args {
 };
 void launch_conv_f32(const ConvF32Args& a, cudaStream_t st);
 // y[r][n] = scale * sum_k h'[k] x[r][n + k + x_off] for n < lout, x zero outside
-// [0, x_len) (x_len < 0: lout + ntaps - 1, valid mode), h' = h or h reversed.
-void launch_fir_f32(const float* x, int64_t x_row, float* y, int64_t y_row, int rows,
-                    const float* taps, int ntaps, int lout, cudaStream_t st, int x_off = 0, int x_len = -1,
-                    int rev = 0, float scale = 1.f);
+// [0, x_len), h' = h or h reversed.
+struct FirArgs {
+  const float* x; int64_t x_row;  // row r at x + r * x_row
+  float* y; int64_t y_row;
+  const float* h; int ntaps;
+  int lout;
+  int x_off, x_len, rev;
+  float scale;
+  const float* x2;      // optional: x - x2 (rows as x) is filtered
+  const float* dscale;  // optional device scalar that the result is multiplied by
+  float* part;          // optional: fir_f32_parts sums of y^2, one per tile
+};
+void launch_fir_f32(const FirArgs& a, int rows, cudaStream_t st);
+int fir_f32_parts(int rows, int lout);
+// Valid mode, y[r][n] = sum_k h[k] x[r][n + k].
+inline FirArgs fir_valid_args(const float* x, int64_t x_row, float* y, int64_t y_row, const float* h, int ntaps,
+                              int lout) {
+  return {x, x_row, y, y_row, h, ntaps, lout, 0, lout + ntaps - 1, 0, 1.f, nullptr, nullptr, nullptr};
+}
+// Its adjoint: y[r][m] = scale * sum_k h[k] x[r][m - k], x of x_len samples, y of x_len + ntaps - 1.
+inline FirArgs fir_adjoint_args(const float* x, int64_t x_row, int x_len, float* y, int64_t y_row, const float* h,
+                                int ntaps, float scale) {
+  return {x, x_row, y, y_row, h, ntaps, x_len + ntaps - 1, -(ntaps - 1), x_len, 1, scale, nullptr, nullptr, nullptr};
+}
 void launch_gap_linear_f32(const float* h, int64_t hb, int64_t hc, int B, int C, int L,
                            const float* w, const float* b, float* out, cudaStream_t st);
 

@@ -70,9 +70,10 @@ void launch_wgrad_tc(const WgradArgs& w, int B, float* partial, float* out, floa
 void launch_standardise(const float* x, int B, int C, int L, const float* mean, const float* istd, float* y,
                         cudaStream_t st);
 // loss = (1 / (B Lr)) sum r^2 with r = g (*) (strain - y_hat) valid (Lr = L - K + 1);
-// e holds B * L floats, r B * Lr, part B.
-void launch_band_loss(const float* strain, const float* y_hat, int B, int L, const float* taps, int K, float* e,
-                      float* r, float* part, float* loss, cudaStream_t st);
+// r holds B * Lr floats, part band_loss_part_floats.
+size_t band_loss_part_floats(int B, int L, int K);
+void launch_band_loss(const float* strain, const float* y_hat, int B, int L, const float* taps, int K, float* r,
+                      float* part, float* loss, cudaStream_t st);
 // dy_hat = dloss * d loss / d y_hat (dloss: device scalar, or null for 1).
 void launch_band_loss_backward(const float* r, int B, int L, const float* taps, int K, const float* dloss,
                                float* dy_hat, cudaStream_t st);

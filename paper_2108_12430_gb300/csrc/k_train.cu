@@ -116,33 +116,13 @@ __global__ void standardise_kernel(const float* __restrict__ x, int64_t n, int C
   }
 }
 
-__global__ void diff_kernel(const float* __restrict__ s, const float* __restrict__ y, int64_t n, float* __restrict__ e) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    e[i] = s[i] - y[i];
-}
-
-// part[b] = sum_n r[b][n]^2 (one CTA per row)
-__global__ void sumsq_rows_kernel(const float* __restrict__ r, int Lr, float* __restrict__ part) {
+// loss = inv_n * sum of the n partial sums (one CTA).
+__global__ void loss_final_kernel(const float* __restrict__ part, int n, float inv_n, float* __restrict__ loss) {
   __shared__ float red[kThreads / 32];
-  const float* row = r + (int64_t)blockIdx.x * Lr;
   float s = 0.f;
-  for (int t = threadIdx.x; t < Lr; t += blockDim.x) s = fmaf(row[t], row[t], s);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) s += part[i];
   s = block_sum(s, red);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-__global__ void loss_final_kernel(const float* __restrict__ part, int B, float inv_n, float* __restrict__ loss) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    float s = 0.f;
-    for (int b = 0; b < B; ++b) s += part[b];
-    *loss = s * inv_n;
-  }
-}
-
-__global__ void scale_by_kernel(float* __restrict__ x, int64_t n, const float* __restrict__ s) {
-  const float v = *s;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    x[i] *= v;
+  if (threadIdx.x == 0) *loss = s * inv_n;
 }
 
 // Adam with bias correction (Kingma & Ba, Algorithm 1), FP32 state.
@@ -226,16 +206,17 @@ void launch_standardise(const float* x, int B, int C, int L, const float* mean, 
   GW_LAUNCH_CHECK();
 }
 
-void launch_band_loss(const float* strain, const float* y_hat, int B, int L, const float* taps, int K, float* e,
-                      float* r, float* part, float* loss, cudaStream_t st) {
-  const int64_t n = (int64_t)B * L;
-  diff_kernel<<<grid_for(n), kThreads, 0, st>>>(strain, y_hat, n, e);
-  GW_LAUNCH_CHECK();
+size_t band_loss_part_floats(int B, int L, int K) { return (size_t)fir_f32_parts(B, L - K + 1); }
+
+void launch_band_loss(const float* strain, const float* y_hat, int B, int L, const float* taps, int K, float* r,
+                      float* part, float* loss, cudaStream_t st) {
   const int Lr = L - K + 1;
-  launch_fir_f32(e, L, r, Lr, B, taps, K, Lr, st);
-  sumsq_rows_kernel<<<B, kThreads, 0, st>>>(r, Lr, part);
-  GW_LAUNCH_CHECK();
-  loss_final_kernel<<<1, 32, 0, st>>>(part, B, 1.f / ((float)B * (float)Lr), loss);
+  FirArgs a = fir_valid_args(strain, L, r, Lr, taps, K, Lr);
+  a.x2 = y_hat;
+  a.part = part;
+  launch_fir_f32(a, B, st);
+  loss_final_kernel<<<1, kThreads, 0, st>>>(part, (int)band_loss_part_floats(B, L, K),
+                                            1.f / ((float)B * (float)Lr), loss);
   GW_LAUNCH_CHECK();
 }
 
@@ -243,12 +224,9 @@ void launch_band_loss_backward(const float* r, int B, int L, const float* taps, 
                                float* dy_hat, cudaStream_t st) {
   const int Lr = L - K + 1;
   // dL/dy_hat[m] = -(2 / N) sum_k g[k] r[m - k]: the FIR's adjoint of r
-  launch_fir_f32(r, Lr, dy_hat, L, B, taps, K, L, st, -(K - 1), Lr, 1, -2.f / ((float)B * (float)Lr));
-  if (dloss) {
-    const int64_t n = (int64_t)B * L;
-    scale_by_kernel<<<grid_for(n), kThreads, 0, st>>>(dy_hat, n, dloss);
-    GW_LAUNCH_CHECK();
-  }
+  FirArgs a = fir_adjoint_args(r, Lr, Lr, dy_hat, L, taps, K, -2.f / ((float)B * (float)Lr));
+  a.dscale = dloss;
+  launch_fir_f32(a, B, st);
 }
 
 void launch_adam_dev(float* p, const float* g, float* m, float* v, int64_t n, int* step, float lr, float b1,

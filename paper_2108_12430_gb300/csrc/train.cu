@@ -573,7 +573,7 @@ int gw_band_loss(gw_fir_t f, const float* strain, const float* y_hat, int B, int
   GW_CHECK_ARG(f && strain && y_hat && loss && r, "NULL argument");
   GW_CHECK_ARG(B >= 1 && L >= f->ntaps, "need B >= 1 and L >= ntaps");
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  const size_t need = ((size_t)B * L + (size_t)B) * sizeof(float);
+  const size_t need = band_loss_part_floats(B, L, f->ntaps) * sizeof(float);
   if (need > f->ws_bytes) {
     GW_CUDA(cudaStreamSynchronize(st));
     if (f->ws) dev_free(f->ctx, f->ws, f->ws_bytes, nullptr);
@@ -582,9 +582,8 @@ int gw_band_loss(gw_fir_t f, const float* strain, const float* y_hat, int B, int
     f->ws = dev_alloc(f->ctx, need, nullptr);
     f->ws_bytes = need;
   }
-  float* e = (float*)f->ws;
   Prof p("band_loss", st);
-  launch_band_loss(strain, y_hat, B, L, f->d_taps, f->ntaps, e, r, e + (size_t)B * L, loss, st);
+  launch_band_loss(strain, y_hat, B, L, f->d_taps, f->ntaps, r, (float*)f->ws, loss, st);
   GW_API_END
 }
 
@@ -604,7 +603,7 @@ int gw_fir_backward(gw_fir_t f, const float* dy, int B, int C, int L_in, float* 
   GW_CHECK_ARG(B >= 1 && C >= 1 && L_in >= f->ntaps, "need B, C >= 1 and L_in >= ntaps");
   const int K = f->ntaps, lout = L_in - K + 1;
   Prof p("fir_bwd", (cudaStream_t)cuda_stream);
-  launch_fir_f32(dy, lout, dx, L_in, B * C, f->d_taps, K, L_in, (cudaStream_t)cuda_stream, -(K - 1), lout, 1, 1.f);
+  launch_fir_f32(fir_adjoint_args(dy, lout, lout, dx, L_in, f->d_taps, K, 1.f), B * C, (cudaStream_t)cuda_stream);
   GW_API_END
 }
 
