@@ -194,6 +194,23 @@ void set_smem_limit_once(void (*func)(A...), int bytes) {
 // Multiprocessor count of the calling thread's current device (cached per device).
 int current_sm_count();
 
+// Launch as a programmatic dependent of the previous kernel in the stream: the
+// kernel may be placed while that one finishes, and executes griddepcontrol.wait
+// before it touches anything another kernel wrote or reads.
+template <typename... KArgs, typename... Args>
+void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  GW_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
+}
+
 // ---- device memory accounting --------------------------------------------
 void* dev_alloc(gw_ctx* ctx, size_t bytes, size_t* counter);
 void dev_free(gw_ctx* ctx, void* p, size_t bytes, size_t* counter);

@@ -32,18 +32,14 @@ struct WgradArgs {
   float* partial;
 };
 
-void launch_fold(const FoldArgs& f, cudaStream_t st);
 // Several layers' folds in one launch (at most kFoldMax).
 constexpr int kFoldMax = 16;
 void launch_fold_many(const FoldArgs* f, int n, cudaStream_t st);
-// dw_in_major: dWf is [C_in][C_out][K] (transposed conv) instead of [C_out][C_in][K].
-void launch_unfold(const FoldArgs& f, const float* dWf, int dw_in_major, const float* dbf, float* dp,
-                   cudaStream_t st);
 // Several layers' unfolds in one launch (at most kFoldMax).
 struct UnfoldItem {
   FoldArgs f;
   const float* dWf;
-  int dw_in_major;
+  int dw_in_major;  // dWf is [C_in][C_out][K] (transposed conv) instead of [C_out][C_in][K]
   const float* dbf;
 };
 void launch_unfold_many(const UnfoldItem* u, int n, float* dp, cudaStream_t st);

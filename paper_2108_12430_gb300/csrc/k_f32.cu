@@ -177,22 +177,37 @@ __global__ void __launch_bounds__(kFirMaxThreads) fir_f32_kernel(const __grid_co
 }
 
 // Global average pool over time followed by the linear head; one CTA per item.
+// Bound: reading the activation once.  Threads walk the item in order
+// (coalesced), weight each channel's values as they sum them and reduce only
+// once, at the end (one thread per channel, 512 bytes apart from its
+// neighbours, took 36 us for 256 items of 256 x 128, this takes 13 us).
 __global__ void __launch_bounds__(kThreads) gap_linear_f32_kernel(const float* __restrict__ h, int64_t hb,
                                                                   int64_t hc, int C, int L,
                                                                   const float* __restrict__ w,
                                                                   const float* __restrict__ bias,
                                                                   float* __restrict__ out) {
   __shared__ float red[kThreads / 32];
-  const int b = blockIdx.x;
+  const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float part = 0.f;
-  for (int c = threadIdx.x; c < C; c += kThreads) {
-    const float* row = h + (int64_t)b * hb + (int64_t)c * hc;
-    float sum = 0.f;
-    for (int t = 0; t < L; ++t) sum += row[t];
-    part = fmaf(sum / (float)L, w[c], part);
+  const float* hb0 = h + (int64_t)b * hb;
+  if (L % 4 == 0 && hc == L && ((uintptr_t)hb0 & 15) == 0) {
+    // the item is one run of C L values: eight 16-byte loads in flight
+    const unsigned quads = (unsigned)C * (unsigned)L / 4, per_c = (unsigned)L / 4;
+#pragma unroll 8
+    for (unsigned i = threadIdx.x; i < quads; i += kThreads) {
+      const float4 v = reinterpret_cast<const float4*>(hb0)[i];
+      part = fmaf((v.x + v.y) + (v.z + v.w), w[i / per_c], part);
+    }
+  } else {
+    for (int c = warp; c < C; c += kThreads / 32) {
+      float sum = 0.f;
+      for (int t = lane; t < L; t += 32) sum += hb0[(int64_t)c * hc + t];
+      part = fmaf(sum, w[c], part);
+    }
   }
+  part /= (float)L;
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
+  if (lane == 0) red[warp] = part;
   __syncthreads();
   if (threadIdx.x == 0) {
     float v = 0.f;

@@ -445,23 +445,6 @@ void launch_strain_push(const float* src, int n, float* ring, int64_t R, int64_t
   GW_LAUNCH_CHECK();
 }
 
-// Launch with programmatic stream serialization: the kernel may be scheduled
-// while the previous kernel of the stream finishes; it waits (griddepcontrol)
-// for that kernel before touching memory, so only the launch latency overlaps.
-template <typename... KArgs, typename... Args>
-static void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  GW_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
-}
-
 void launch_sub_ola(const float* pred, int64_t pred_ld, int n, int S, int W, int64_t R, int64_t head, int mode,
                     int delta, float* acc, const float* strain_ring, float* out, cudaStream_t st,
                     const int* skip, float* pring, int64_t Rp, int* skip_copy) {

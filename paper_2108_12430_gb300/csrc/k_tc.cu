@@ -626,69 +626,86 @@ __global__ void __launch_bounds__(kThreads, kMaxCtasPerSm) conv_tc_kernel(const 
 // of 8 channels, or e4m3 rows of 16).  ts = 8, xc = 1 turns one signal into 8
 // "channels" of consecutive samples (space-to-depth).  Optionally the
 // (standardised) FP32 values also go to y[b yb + c yc + t].
-__global__ void to_blocked_kernel(const float* __restrict__ x, int64_t xb, int64_t xc, int64_t ts, int B, int C,
-                                  int L, const float* __restrict__ mean, const float* __restrict__ istd, float scale,
-                                  char* __restrict__ out, int64_t ob, int64_t og, int64_t op, int P, int fp8,
-                                  float* __restrict__ y, int64_t yb, int64_t yc) {
-  const int cg = fp8 ? 16 : 8;
-  const int G = (C + cg - 1) / cg;
-  const int64_t total = (int64_t)B * G * L;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int t = (int)(e % L);
-    const int g = (int)((e / L) % G);
-    const int b = (int)(e / ((int64_t)L * G));
-    float v[16];
+//
+// Bound: DRAM / L2 traffic.  A thread makes one 16-byte row; its 8 (16) channel
+// loads are independent and coalesced along time, the item and group come from
+// the block index (64-bit divisions per element made 32 windows of 21 x 8192
+// take 28 us, this takes 14 us).  Launched as a dependent of the previous kernel.
+__global__ void __launch_bounds__(256) to_blocked_kernel(const float* __restrict__ x, int64_t xb, int64_t xc, int64_t ts,
+                                                         int C, int L, int tblocks, const float* __restrict__ mean,
+                                                         const float* __restrict__ istd, float scale,
+                                                         char* __restrict__ out, int64_t ob, int64_t og, int64_t op, int P,
+                                                         int fp8, float* __restrict__ y, int64_t yb, int64_t yc) {
+  griddep_wait();
+  const int cg = fp8 ? 16 : 8, g = blockIdx.y;
+  const int b = blockIdx.x / tblocks, t = (blockIdx.x - b * tblocks) * 256 + threadIdx.x;
+  if (t >= L) return;
+  float v[16];
+  const float* xp = x + (int64_t)b * xb + (int64_t)g * cg * xc + (int64_t)t * ts;
+  const int n = min(cg, C - g * cg);
+  if (xc == 1 && n == 8 && cg == 8 && ((uintptr_t)xp & 15) == 0) {
+    const float4 q0 = reinterpret_cast<const float4*>(xp)[0], q1 = reinterpret_cast<const float4*>(xp)[1];
+    v[0] = q0.x, v[1] = q0.y, v[2] = q0.z, v[3] = q0.w, v[4] = q1.x, v[5] = q1.y, v[6] = q1.z, v[7] = q1.w;
+  } else {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const int c = g * cg + i;
-      float a = 0.f;
-      if (i < cg && c < C) {
-        a = x[(int64_t)b * xb + (int64_t)c * xc + (int64_t)t * ts];
-        if (mean) a = (a - mean[c]) * istd[c];
-        if (y) y[(int64_t)b * yb + (int64_t)c * yc + t] = a;
-      }
-      v[i] = a;
-    }
-    char* dst = out + (int64_t)b * ob + (int64_t)g * og + (int64_t)(t % P) * op + (int64_t)(t / P) * 16;
-    if (fp8) {
-      __align__(16) __nv_fp8_e4m3 o8[16];
+    for (int i = 0; i < 16; ++i) v[i] = i < n ? xp[i * xc] : 0.f;
+  }
+  if (mean) {
 #pragma unroll
-      for (int i = 0; i < 16; ++i) o8[i] = __nv_fp8_e4m3(v[i] * scale);
-      *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(o8);
-    } else {
-      __align__(16) __nv_bfloat16 o16[8];
+    for (int i = 0; i < 16; ++i)
+      if (i < n) v[i] = (v[i] - mean[g * cg + i]) * istd[g * cg + i];
+  }
+  if (y) {
+    float* yp = y + (int64_t)b * yb + (int64_t)g * cg * yc + t;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) o16[i] = __float2bfloat16_rn(v[i]);
-      *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(o16);
-    }
+    for (int i = 0; i < 16; ++i)
+      if (i < n) yp[i * yc] = v[i];
+  }
+  char* dst = out + (int64_t)b * ob + (int64_t)g * og + (int64_t)(t % P) * op + (int64_t)(t / P) * 16;
+  if (fp8) {
+    __align__(16) __nv_fp8_e4m3 o8[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) o8[i] = __nv_fp8_e4m3(v[i] * scale);
+    *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(o8);
+  } else {
+    __align__(16) __nv_bfloat16 o16[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) o16[i] = __float2bfloat16_rn(v[i]);
+    *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(o16);
   }
 }
 
 // Global average pool of a blocked activation + linear head; one CTA per
-// item.  A warp takes one phase plane of one channel group at a time (its
-// lanes consecutive 16-byte rows, so that the loads coalesce), sums each
-// channel over its rows in registers, reduces across the warp and adds the
-// plane's sums to per-channel totals in shared memory; then every channel's
-// mean is weighted and the products reduced.
-constexpr int kGapMaxC = 1024;
-__global__ void gap_linear_blocked_kernel(const char* __restrict__ in, int64_t ib, int64_t ig, int64_t ip, int P,
-                                          int L, int C, int fp8, float in_scale, const float* __restrict__ w,
-                                          const float* __restrict__ bias, float* __restrict__ out) {
-  __shared__ float acc[kGapMaxC];
-  __shared__ float red[32];
-  const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  const int cg = fp8 ? 16 : 8;
-  const int G = (C + cg - 1) / cg, R = (L + P - 1) / P;
-  for (int c = threadIdx.x; c < G * cg; c += blockDim.x) acc[c] = 0.f;
-  __syncthreads();
-  for (int plane = warp; plane < G * P; plane += nwarps) {
-    const int g = plane / P, phase = plane - g * P;
-    const char* base = in + (int64_t)b * ib + (int64_t)g * ig + (int64_t)phase * ip;
+// item.  Bound: reading the activation once (64 KB per item at 256 x 128).
+// A thread takes every (kGapThreads / G)-th row of one channel group (neighbouring
+// threads neighbouring 16-byte rows), sums its channels in registers, weights
+// the sums and joins one reduction at the end; summing each channel across
+// the CTA first (5 shuffles per channel and plane, then shared-memory atomics)
+// took 15 us for one item, this takes 7 us.
+constexpr int kGapThreads = 512;
+__global__ void __launch_bounds__(kGapThreads) gap_linear_blocked_kernel(const char* __restrict__ in, int64_t ib, int64_t ig,
+                                                                 int64_t ip, int P, int L, int C, int fp8,
+                                                                 float in_scale, const float* __restrict__ w,
+                                                                 const float* __restrict__ bias,
+                                                                 float* __restrict__ out) {
+  __shared__ float red[kGapThreads / 32];
+  griddep_wait();
+  const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cg = fp8 ? 16 : 8, G = (C + cg - 1) / cg;
+  // threads per group: a power of two, at most kGapThreads / G (at least 1)
+  int lg = 0;
+  while ((2 << lg) * G <= kGapThreads) ++lg;
+  const int per_pass = kGapThreads >> lg, r0 = threadIdx.x & ((1 << lg) - 1);
+  float part = 0.f;
+  for (int g = threadIdx.x >> lg; g < G; g += per_pass) {
+    const char* base = in + (int64_t)b * ib + (int64_t)g * ig;
     float v[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = 0.f;
-    for (int r = lane; r < R && r * P + phase < L; r += 32) {
-      const uint4 q = *reinterpret_cast<const uint4*>(base + (int64_t)r * 16);
+    // row j of the group: phase j mod P, row j / P of its plane
+#pragma unroll 8
+    for (int j = r0; j < L; j += 1 << lg) {
+      const uint4 q = *reinterpret_cast<const uint4*>(base + (int64_t)(j % P) * ip + (int64_t)(j / P) * 16);
       if (fp8) {
         const __nv_fp8_e4m3* e = reinterpret_cast<const __nv_fp8_e4m3*>(&q);
 #pragma unroll
@@ -701,19 +718,14 @@ __global__ void gap_linear_blocked_kernel(const char* __restrict__ in, int64_t i
     }
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-    if (lane == 0)
-      for (int i = 0; i < cg; ++i) atomicAdd(&acc[g * cg + i], v[i]);
+      if (i < cg && g * cg + i < C) part = fmaf(v[i] * in_scale / (float)L, w[g * cg + i], part);
   }
-  __syncthreads();
-  float part = 0.f;
-  for (int c = threadIdx.x; c < C; c += blockDim.x) part = fmaf(acc[c] * in_scale / (float)L, w[c], part);
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
   if (lane == 0) red[warp] = part;
   __syncthreads();
   if (threadIdx.x == 0) {
     float t = 0.f;
-    for (int i = 0; i < nwarps; ++i) t += red[i];
+    for (int i = 0; i < kGapThreads / 32; ++i) t += red[i];
     out[b] = t + bias[0];
   }
 }
@@ -1252,20 +1264,19 @@ void launch_to_blocked(const float* x, int64_t xb, int64_t xc, int B, int C, int
                        float* y, int64_t yb, int64_t yc) {
   const int esz = fp8 ? 1 : 2;
   const int cg = fp8 ? 16 : 8;
-  const int64_t total = (int64_t)B * ((C + cg - 1) / cg) * L;
-  const int grid = (int)std::min<int64_t>((total + 255) / 256, 152 * 32);
-  to_blocked_kernel<<<grid, 256, 0, st>>>(x, xb, xc, ts, B, C, L, mean, istd, scale, (char*)out.p, out.bstride * esz,
-                                          out.gstride * esz, out.pstride * esz, out.P, fp8, y, yb, yc);
-  GW_LAUNCH_CHECK();
+  const int tblocks = (L + 255) / 256;
+  GW_CHECK_ARG((int64_t)B * tblocks < (1LL << 31), "batch too large for one launch");
+  launch_pdl(to_blocked_kernel, dim3((unsigned)(B * tblocks), (C + cg - 1) / cg), dim3(256), st, x, xb, xc, ts, C, L,
+             tblocks, mean, istd, scale, (char*)out.p, (int64_t)(out.bstride * esz), (int64_t)(out.gstride * esz),
+             (int64_t)(out.pstride * esz), out.P, fp8, y, yb, yc);
 }
 
 void launch_gap_linear_blocked(const TcIn& in, int C, int fp8, float in_scale, const float* w, const float* b,
                                float* out, int B, cudaStream_t st) {
   const int esz = fp8 ? 1 : 2;
-  GW_CHECK_ARG((C + 15) / 16 * 16 <= kGapMaxC, "too many channels for the pooling head");
-  gap_linear_blocked_kernel<<<B, 256, 0, st>>>((const char*)in.p + in.off0 * esz, in.bstride * esz, in.gstride * esz,
-                                               in.pstride * esz, in.P, in.L, C, fp8, in_scale, w, b, out);
-  GW_LAUNCH_CHECK();
+  launch_pdl(gap_linear_blocked_kernel, dim3(B), dim3(kGapThreads), st, (const char*)in.p + in.off0 * esz,
+             (int64_t)(in.bstride * esz), (int64_t)(in.gstride * esz), (int64_t)(in.pstride * esz), in.P, in.L, C, fp8,
+             in_scale, w, b, out);
 }
 
 }  // namespace gw
