@@ -39,6 +39,7 @@
 
 #include <algorithm>
 #include <set>
+#include <type_traits>
 
 #include "gw_internal.h"
 #include "tc_ptx.h"
@@ -103,7 +104,7 @@ struct TcParams {
   float out_scale;
   const char* res;
   int64_t res_b, res_g, res_p;  // bytes
-  int res_P, res_fp8;
+  int res_P;
   float res_scale;
   int* err;
   int coutp_log, out_P_log, res_P_log;  // power-of-two shifts for the epilogue addressing
@@ -169,9 +170,18 @@ __host__ __device__ __forceinline__ uint32_t slice_off(uint32_t code, int P, int
   return ((g * (uint32_t)P + phi) * (uint32_t)rows + dd) * 16u;
 }
 
-// kFull: the FP32 [B][C][L] output mode of the training path is compiled only
-// into its own instantiation, so the inference kernel's epilogue is unchanged.
-template <bool kFull>
+// One instantiation per kind of epilogue, so that each keeps only its own
+// values in registers: bf16 rows (also the FP32 prediction and the FIR's
+// samples), the training path's FP32 [B][C][L], bf16 rows plus a residual, and
+// e4m3 (scales, e4m3 output) without and with a residual.  What bounded the
+// epilogues was latency and narrow accesses: a residual cost one L2 round trip
+// per 8 channels (block 1's second conv, 256 items: 28.6 us, 19.9 us with the
+// rows fetched a chunk ahead), e4m3 rows went out 8 bytes at a time from scalar
+// conversions (28.8 -> 18.5 us), FP32 planes 4 bytes at a time with 2-byte
+// stores of the blocked copy (32 windows of 8192, 8 -> 16 channels: 26.1 ->
+// 12.9 us).
+enum { kEpiPlain = 0, kEpiFull = 1, kEpiRes = 2, kEpiFp8 = 3, kEpiFp8Res = 4 };
+template <int kEpi>
 __global__ void __launch_bounds__(kThreads, kMaxCtasPerSm) conv_tc_kernel(const TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
@@ -460,11 +470,34 @@ __global__ void __launch_bounds__(kThreads, kMaxCtasPerSm) conv_tc_kernel(const 
     const int quarter = warp & 3;          // TMEM lanes this warp may access
     const int col_half = (warp - 2) >> 2;  // first 32-column chunk it drains (then every kEpiWarps / 4-th)
     const int row = quarter * 32 + lane;
-    const bool plain = !kFull && !p.fp32_single && !p.fp32_d2s && !p.fp8_out && !p.res && !p.wscale;
+    constexpr bool kFull = kEpi == kEpiFull, kRes = kEpi == kEpiRes || kEpi == kEpiFp8Res;
+    constexpr bool kFp8 = kEpi == kEpiFp8 || kEpi == kEpiFp8Res;
+    const int out_mask = p.out_P - 1, res_mask = p.res_P - 1, n_chunk = p.ncol / 32;
+    // Residual of the 32 columns of chunk j (bf16: four 16-byte rows of 8
+    // channels; e4m3: two of 16).  The loads go out a chunk ahead -- the first
+    // ones before the tile's accumulator is ready -- so that their latency
+    // overlaps the MMAs and the previous chunk's arithmetic.
+    constexpr int kResRows = kRes ? (kFp8 ? 2 : 4) : 1;
+    uint4 rq[kResRows];
+    auto load_res = [&](int h, int b, int m, int jg) {
+      constexpr int step = kFp8 ? 16 : 8, lg = kFp8 ? 4 : 3;
+      const int n0 = jg * 32 + h * step;
+      const int sg = n0 >> p.coutp_log, o0 = n0 & (p.coutp - 1), u = p.Q * m + sg;
+      rq[h] = make_uint4(0u, 0u, 0u, 0u);
+      if (m < p.mout && sg < p.Q && o0 < p.cout && u < p.lout)
+        rq[h] = *reinterpret_cast<const uint4*>(p.res + (int64_t)b * p.res_b + (int64_t)(o0 >> lg) * p.res_g +
+                                                (int64_t)(u & res_mask) * p.res_p + (int64_t)(u >> p.res_P_log) * 16);
+    };
     griddep_wait();  // outputs and residuals are shared with the previous kernels
     int i = 0;
     for (int t = blockIdx.x; t < p.n_tiles; t += gridDim.x, ++i) {
       const int s = i & 1, k = i >> 1;
+      int b, m0, sl;
+      tile_coords(p, t, b, m0, sl);
+      if constexpr (kRes) {
+#pragma unroll
+        for (int h = 0; h < kResRows; ++h) load_res(h, b, m0 + row, sl * n_chunk + col_half);
+      }
       // One warp polls the accumulator barrier; the other seven sleep in the
       // named barrier instead of spinning on issue slots that the MMA thread,
       // the producer and the other CTA on the SM need.
@@ -472,71 +505,113 @@ __global__ void __launch_bounds__(kThreads, kMaxCtasPerSm) conv_tc_kernel(const 
       if (warp == 2) ok = mbar_wait(bar(acc_full + s), (uint32_t)k & 1u, abort_flag, p.err, kErrWaitAcc);
       if (!epi_bar_and(ok)) break;
       tc_fence_after();
-      int b, m0, sl;
-      tile_coords(p, t, b, m0, sl);
       char* const outb = p.out + (int64_t)b * p.out_b;
-      const char* const resb = p.res ? p.res + (int64_t)b * p.res_b : nullptr;
-      const int out_mask = p.out_P - 1, res_mask = p.res_P - 1;
       for (int mt = 0; mt < p.MT; ++mt) {
         const int m = m0 + mt * 128 + row;
         const bool valid = m < p.mout;
-        for (int j = col_half; j < p.ncol / 32; j += kEpiWarps / 4) {
+        for (int j = col_half; j < n_chunk; j += kEpiWarps / 4) {
           float v[32];
           tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((s * p.MT + mt) * p.ncol + j * 32), v);
-          if (!valid) continue;
-          const int jg = sl * (p.ncol / 32) + j;  // chunk index among all npad columns
-          if (plain) {
-            // bf16 out, no residual, no FP8 scale: 4 groups of 8 channels,
-            // straight-line, bias as float4 pairs, no per-group branches
-            // (the common DeepClean / BBHnet case; invalid groups are those
-            // past Q, C_out or the output length, known per column / row)
-            const int n_base = jg * 32;
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              const int n0 = n_base + h * 8;
-              const int sg = n0 >> p.coutp_log, o0 = n0 & (p.coutp - 1);
-              const int u = p.Q * m + sg;
-              const float4 b0 = *reinterpret_cast<const float4*>(s_bias + o0);
-              const float4 b1 = *reinterpret_cast<const float4*>(s_bias + o0 + 4);
-              const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-              __align__(16) __nv_bfloat162 o16[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e)
-                o16[e] = __floats2bfloat162_rn(act_fn(v[h * 8 + 2 * e] + bb[2 * e], p.act),
-                                               act_fn(v[h * 8 + 2 * e + 1] + bb[2 * e + 1], p.act));
-              if (sg < p.Q && o0 < p.cout && u < p.lout) {
-                char* op = outb + (int64_t)(o0 >> 3) * p.out_g + (int64_t)(u & out_mask) * p.out_p +
-                           (int64_t)(u >> p.out_P_log) * 16;
-                *reinterpret_cast<uint4*>(op) = *reinterpret_cast<const uint4*>(o16);
-              }
-            }
-            continue;
-          }
-          if (kFull) {
+          const int jg = sl * n_chunk + j;  // chunk index among all npad columns
+          if constexpr (kFull) {
             // FP32 [B][C][L] (training): bias, activation, optionally times the
-            // derivative of the activation whose output is gy
+            // derivative of the activation whose output is gy; and optionally
+            // the same values in the next layer's blocked BF16 layout
+            if (!valid) continue;
+            float* outf = reinterpret_cast<float*>(outb);
+            const int64_t out_c = p.out_g / 4;
             const float* gyb = p.gy ? p.gy + (int64_t)b * p.gy_b : nullptr;
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              const int n = jg * 32 + e;
-              const int sg = n >> p.coutp_log, o = n & (p.coutp - 1);
-              const int u = p.Q * m + sg;
-              if (sg >= p.Q || o >= p.cout || u >= p.lout) continue;
-              float val = act_fn(v[e] + s_bias[o], p.act);
+            // a thread's columns: `np` consecutive positions of coutp channels
+            // (32 columns hold 4 x 8, 2 x 16, or 32 channels of one position)
+            const int n0 = jg * 32, sg0 = n0 >> p.coutp_log, o0 = n0 & (p.coutp - 1), u0 = p.Q * m + sg0;
+            auto positions = [&](auto npc) {
+              constexpr int NP = decltype(npc)::value, NC = 32 / NP;
+              typedef typename std::conditional<NP == 4, float4, typename std::conditional<NP == 2, float2, float>::type>::type V;
+              const int left = min(p.lout - u0, p.Q - sg0);  // positions of this chunk that exist
+              if (left <= 0) return;
+              const bool vec = NP > 1 && left >= NP && ((uintptr_t)(outf + u0) & (4 * NP - 1)) == 0 && out_c % NP == 0 &&
+                               (!gyb || (((uintptr_t)(gyb + u0) & (4 * NP - 1)) == 0 && p.gy_c % NP == 0));
               if (gyb) {
-                const float a = gyb[(int64_t)o * p.gy_c + u];
-                val *= p.gact == ACT_TANH ? 1.f - a * a : (a > 0.f ? 1.f : 0.f);
+                // derivative factors of a quarter of the chunk's columns at a time
+#pragma unroll
+                for (int c0 = 0; c0 < NC; c0 += NC / 4) {
+                  float a[8];
+#pragma unroll
+                  for (int c = 0; c < NC / 4; ++c) {
+                    const int o = o0 + c0 + c;
+                    if (vec && o < p.cout) {
+                      const V q = *reinterpret_cast<const V*>(gyb + (int64_t)o * p.gy_c + u0);
+#pragma unroll
+                      for (int e = 0; e < NP; ++e) a[c * NP + e] = reinterpret_cast<const float*>(&q)[e];
+                    } else {
+#pragma unroll
+                      for (int e = 0; e < NP; ++e)
+                        a[c * NP + e] = (o < p.cout && e < left) ? gyb[(int64_t)o * p.gy_c + u0 + e] : 0.f;
+                    }
+                  }
+#pragma unroll
+                  for (int c = 0; c < NC / 4; ++c)
+#pragma unroll
+                    for (int e = 0; e < NP; ++e) {
+                      const float av = a[c * NP + e];
+                      float& x = v[e * NC + c0 + c];
+                      x = act_fn(x + s_bias[o0 + c0 + c], p.act);
+                      x *= p.gact == ACT_TANH ? 1.f - av * av : (av > 0.f ? 1.f : 0.f);
+                    }
+                }
+              } else {
+#pragma unroll
+                for (int c = 0; c < NC; ++c)
+#pragma unroll
+                  for (int e = 0; e < NP; ++e) v[e * NC + c] = act_fn(v[e * NC + c] + s_bias[o0 + c], p.act);
               }
-              reinterpret_cast<float*>(outb + (int64_t)o * p.out_g)[u] = val;
-              if (p.blk)
-                *reinterpret_cast<__nv_bfloat16*>(p.blk + (int64_t)b * p.blk_b + (int64_t)(o >> 3) * p.blk_g +
-                                                  (int64_t)(u & ((1 << p.blk_P_log) - 1)) * p.blk_p +
-                                                  (int64_t)(u >> p.blk_P_log) * 16 + (o & 7) * 2) =
-                    __float2bfloat16_rn(val);
-            }
+#pragma unroll
+              for (int c = 0; c < NC; ++c) {
+                const int o = o0 + c;
+                if (o >= p.cout) continue;
+                float* dst = outf + (int64_t)o * out_c + u0;
+                if (vec) {
+                  V q;
+#pragma unroll
+                  for (int e = 0; e < NP; ++e) reinterpret_cast<float*>(&q)[e] = v[e * NC + c];
+                  *reinterpret_cast<V*>(dst) = q;
+                } else {
+#pragma unroll
+                  for (int e = 0; e < NP; ++e)
+                    if (e < left) dst[e] = v[e * NC + c];
+                }
+              }
+              if (p.blk) {
+                char* blkb = p.blk + (int64_t)b * p.blk_b;
+                const int mask = (1 << p.blk_P_log) - 1;
+#pragma unroll
+                for (int e = 0; e < NP; ++e) {
+                  const int u = u0 + e;
+                  if (e >= left) continue;
+                  char* row8 = blkb + (int64_t)(u & mask) * p.blk_p + (int64_t)(u >> p.blk_P_log) * 16;
+#pragma unroll
+                  for (int c = 0; c < NC; c += 8) {
+                    if (o0 + c >= p.cout) continue;
+                    __align__(16) __nv_bfloat162 q[4];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h)
+                      q[h] = __floats2bfloat162_rn(v[e * NC + c + 2 * h],
+                                                   v[e * NC + c + 2 * h + 1]);
+                    *reinterpret_cast<uint4*>(row8 + (int64_t)((o0 + c) >> 3) * p.blk_g) = *reinterpret_cast<const uint4*>(q);
+                  }
+                }
+              }
+            };
+            if (p.coutp_log == 3)
+              positions(std::integral_constant<int, 4>());
+            else if (p.coutp_log == 4)
+              positions(std::integral_constant<int, 2>());
+            else
+              positions(std::integral_constant<int, 1>());
             continue;
           }
-          if (p.fp32_single) {
+          if (kEpi == kEpiPlain && p.fp32_single) {
+            if (!valid) continue;
             // column n = sigma: output position Q m + sigma, channel 0
             float* y = reinterpret_cast<float*>(outb);
             const float bias = s_bias[0];
@@ -558,56 +633,90 @@ __global__ void __launch_bounds__(kThreads, kMaxCtasPerSm) conv_tc_kernel(const 
             }
             continue;
           }
+          // bf16 or e4m3 rows: dequantise (e4m3 operands), bias, residual,
+          // activation, straight-line per 8 (16) channels; invalid groups are those
+          // past Q, C_out or the output length, known per column / row.  Each row
+          // of the next chunk's residual is fetched as soon as this chunk's has
+          // been used.
+          const bool more = j + kEpiWarps / 4 < n_chunk, next = more || mt + 1 < p.MT;
+          const int m_next = more ? m : m + 128, j_next = sl * n_chunk + (more ? j + kEpiWarps / 4 : col_half);
+          const int n_base = jg * 32;
 #pragma unroll
           for (int h = 0; h < 4; ++h) {
-            const int n0 = jg * 32 + h * 8;
-            const int sg = n0 >> p.coutp_log, o0 = n0 & (p.coutp - 1);
-            const int u = p.Q * m + sg;
-            if (sg >= p.Q || o0 >= p.cout || u >= p.lout) continue;
-            float x[8];
+            const int o0 = (n_base + h * 8) & (p.coutp - 1);
+            const float4 b0 = *reinterpret_cast<const float4*>(s_bias + o0);
+            const float4 b1 = *reinterpret_cast<const float4*>(s_bias + o0 + 4);
+            const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+            float* x = v + h * 8;
+            if (kFp8 && p.wscale) {
+              const float4 s0 = *reinterpret_cast<const float4*>(s_scale + o0);
+              const float4 s1 = *reinterpret_cast<const float4*>(s_scale + o0 + 4);
+              const float ss[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const int o = o0 + e;
-              x[e] = o < p.cout ? fmaf(v[h * 8 + e], s_scale[o], s_bias[o]) : 0.f;
+              for (int e = 0; e < 8; ++e) x[e] = fmaf(x[e], ss[e], bb[e]);
+            } else {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) x[e] += bb[e];
             }
-            if (resb) {
-              if (p.res_fp8) {
-                const char* rp = resb + (int64_t)(o0 >> 4) * p.res_g + (int64_t)(u & res_mask) * p.res_p +
-                                 (int64_t)(u >> p.res_P_log) * 16 + (o0 & 15);
-                const uint2 rv = *reinterpret_cast<const uint2*>(rp);
-                const __nv_fp8_e4m3* r8 = reinterpret_cast<const __nv_fp8_e4m3*>(&rv);
+            if constexpr (kRes) {
+              if constexpr (kFp8) {
+                const uint4& rv = rq[h >> 1];
+                const uint32_t w2[2] = {(h & 1) ? rv.z : rv.x, (h & 1) ? rv.w : rv.y};
 #pragma unroll
-                for (int e = 0; e < 8; ++e) x[e] += float(r8[e]) * p.res_scale;
+                for (int e = 0; e < 4; ++e) {
+                  const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2(
+                      (__nv_fp8x2_storage_t)((w2[e >> 1] >> ((e & 1) * 16)) & 0xFFFFu), __NV_E4M3);
+                  const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hr));
+                  x[2 * e] = fmaf(f.x, p.res_scale, x[2 * e]);
+                  x[2 * e + 1] = fmaf(f.y, p.res_scale, x[2 * e + 1]);
+                }
               } else {
-                const char* rp = resb + (int64_t)(o0 >> 3) * p.res_g + (int64_t)(u & res_mask) * p.res_p +
-                                 (int64_t)(u >> p.res_P_log) * 16;
-                const uint4 rv = *reinterpret_cast<const uint4*>(rp);
-                const __nv_bfloat16* r16 = reinterpret_cast<const __nv_bfloat16*>(&rv);
+                const uint32_t w4[4] = {rq[h].x, rq[h].y, rq[h].z, rq[h].w};
 #pragma unroll
-                for (int e = 0; e < 8; ++e) x[e] += __bfloat162float(r16[e]);
+                for (int e = 0; e < 4; ++e) {
+                  const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w4[e]));
+                  x[2 * e] += f.x;
+                  x[2 * e + 1] += f.y;
+                }
               }
+              if (next && (!kFp8 || (h & 1))) load_res(kFp8 ? h >> 1 : h, b, m_next, j_next);
             }
 #pragma unroll
             for (int e = 0; e < 8; ++e) x[e] = act_fn(x[e], p.act);
-            if (p.fp32_d2s) {
+            if (!(kFp8 && p.fp8_out) && !(kEpi == kEpiPlain && p.fp32_d2s)) {
+              const int sg = (n_base + h * 8) >> p.coutp_log, u = p.Q * m + sg;
+              __align__(16) __nv_bfloat162 o16[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) o16[e] = __floats2bfloat162_rn(x[2 * e], x[2 * e + 1]);
+              if (valid && sg < p.Q && o0 < p.cout && u < p.lout)
+                *reinterpret_cast<uint4*>(outb + (int64_t)(o0 >> 3) * p.out_g + (int64_t)(u & out_mask) * p.out_p +
+                                          (int64_t)(u >> p.out_P_log) * 16) = *reinterpret_cast<const uint4*>(o16);
+            }
+          }
+          if (!valid) continue;
+          if (kEpi == kEpiPlain && p.fp32_d2s) {
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
               // depth-to-space: channel o of position u is output sample 8 u + o
+              const int sg = (n_base + h * 8) >> p.coutp_log, u = p.Q * m + sg;
+              if (sg >= p.Q || u >= p.lout) continue;
               float4* op = reinterpret_cast<float4*>(outb + (int64_t)u * 32);
-              op[0] = make_float4(x[0], x[1], x[2], x[3]);
-              op[1] = make_float4(x[4], x[5], x[6], x[7]);
-            } else if (p.fp8_out) {
-              __align__(8) __nv_fp8_e4m3 o8[8];
+              op[0] = make_float4(v[h * 8], v[h * 8 + 1], v[h * 8 + 2], v[h * 8 + 3]);
+              op[1] = make_float4(v[h * 8 + 4], v[h * 8 + 5], v[h * 8 + 6], v[h * 8 + 7]);
+            }
+          } else if (kFp8 && p.fp8_out) {
 #pragma unroll
-              for (int e = 0; e < 8; ++e) o8[e] = __nv_fp8_e4m3(x[e] * p.out_scale);
-              char* op = outb + (int64_t)(o0 >> 4) * p.out_g + (int64_t)(u & out_mask) * p.out_p +
-                         (int64_t)(u >> p.out_P_log) * 16 + (o0 & 15);
-              *reinterpret_cast<uint2*>(op) = *reinterpret_cast<const uint2*>(o8);
-            } else {
-              __align__(16) __nv_bfloat16 o16[8];
+            for (int h = 0; h < 2; ++h) {
+              const int n0 = n_base + h * 16;
+              const int sg = n0 >> p.coutp_log, o0 = n0 & (p.coutp - 1), u = p.Q * m + sg;
+              if (sg >= p.Q || o0 >= p.cout || u >= p.lout) continue;
+              __align__(16) __nv_fp8x2_storage_t o8[8];
 #pragma unroll
-              for (int e = 0; e < 8; ++e) o16[e] = __float2bfloat16_rn(x[e]);
-              char* op = outb + (int64_t)(o0 >> 3) * p.out_g + (int64_t)(u & out_mask) * p.out_p +
-                         (int64_t)(u >> p.out_P_log) * 16;
-              *reinterpret_cast<uint4*>(op) = *reinterpret_cast<const uint4*>(o16);
+              for (int e = 0; e < 8; ++e)
+                o8[e] = __nv_cvt_float2_to_fp8x2(make_float2(v[h * 16 + 2 * e] * p.out_scale, v[h * 16 + 2 * e + 1] * p.out_scale),
+                                                 __NV_SATFINITE, __NV_E4M3);
+              *reinterpret_cast<uint4*>(outb + (int64_t)(o0 >> 4) * p.out_g + (int64_t)(u & out_mask) * p.out_p +
+                                        (int64_t)(u >> p.out_P_log) * 16) = *reinterpret_cast<const uint4*>(o8);
             }
           }
         }
@@ -1183,6 +1292,10 @@ static void plan_conv_tc(TcParams& q, const LayerDev& L, bool fp8, const TcIn& i
   q.out_P = out.P;
   q.fp32_single = out.fp32_single;
   q.fp8_out = out.fp8_out;
+  GW_CHECK_ARG(!(out.fp8_out || (out.res && fp8)) || (L.coutp % 16 == 0 && s.cout % 16 == 0),
+               "e4m3 rows hold 16 channels of one position");
+  GW_CHECK_ARG(!out.res || s.cout % 8 == 0, "residual rows hold 8 channels");
+  GW_CHECK_ARG(!out.fp32_full || L.coutp >= 8, "FP32 [B][C][L] output: at least 8 columns per position");
   q.out_scale = L.out_scale;
   q.res = (const char*)out.res;
   const int resz = fp8 ? 1 : 2;
@@ -1190,7 +1303,6 @@ static void plan_conv_tc(TcParams& q, const LayerDev& L, bool fp8, const TcIn& i
   q.res_g = out.rgstride * resz;
   q.res_p = out.rpstride * resz;
   q.res_P = out.rP ? out.rP : 1;
-  q.res_fp8 = fp8 ? 1 : 0;
   q.res_scale = fp8 ? 1.0f / L.out_scale : 1.0f;
   q.err = err;
   auto log2_exact = [](int v, const char* what) {
@@ -1238,8 +1350,6 @@ void launch_conv_tc(const LayerDev& L, const TcIn& in, int lout, const TcOut& ou
   dim3 grid;
   plan_conv_tc(q, L, L.wscale != nullptr, in, lout, out, err, &smem, &grid, B, current_sm_count());
   q.stall_test = tc_take_stall_test() ? 1 : 0;
-  set_smem_limit_once(conv_tc_kernel<false>, 227 * 1024);
-  set_smem_limit_once(conv_tc_kernel<true>, 227 * 1024);
   // programmatic stream serialisation: this launch may begin (set-up, weight
   // loads) while the previous kernel in the stream runs; the kernel waits on
   // griddepcontrol before touching the previous kernels' data
@@ -1253,10 +1363,15 @@ void launch_conv_tc(const LayerDev& L, const TcIn& in, int lout, const TcOut& ou
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  auto kernel = conv_tc_kernel<kEpiPlain>;
   if (q.fp32_full)
-    GW_CUDA(cudaLaunchKernelEx(&cfg, conv_tc_kernel<true>, q));
-  else
-    GW_CUDA(cudaLaunchKernelEx(&cfg, conv_tc_kernel<false>, q));
+    kernel = conv_tc_kernel<kEpiFull>;
+  else if (q.fp8_out || q.wscale)
+    kernel = q.res ? conv_tc_kernel<kEpiFp8Res> : conv_tc_kernel<kEpiFp8>;
+  else if (q.res)
+    kernel = conv_tc_kernel<kEpiRes>;
+  set_smem_limit_once(kernel, 227 * 1024);
+  GW_CUDA(cudaLaunchKernelEx(&cfg, kernel, q));
 }
 
 void launch_to_blocked(const float* x, int64_t xb, int64_t xc, int B, int C, int L, const float* mean,
