@@ -57,12 +57,18 @@ size_t wgrad_f32_partial_floats(const WgradArgs& w, int B);
 WgradReduceItem launch_wgrad_f32(const WgradArgs& w, int B, float* out, float* db, cudaStream_t st);
 void launch_wgrad_reduce(const WgradReduceItem* items, int n, cudaStream_t st);
 // The same weight gradient on the tensor cores (BF16 operands, FP32
-// accumulation; k_wgrad_tc.cu): out gets NA * NC * K floats and, with
-// w.bias, db the bias gradient (NA floats for bias 1, NC for bias 2); partial
-// must hold wgrad_tc_partial_floats(w, B); err receives a bounded wait's give-up.
+// accumulation; k_wgrad_tc.cu): w.partial must hold wgrad_tc_partial_floats;
+// err receives a bounded wait's give-up.  Returns what launch_wgrad_tc_reduce
+// needs to add the partials into out (NA * NC * K floats) and, with w.bias, db.
+struct WgradTcReduceItem {
+  const float* partial;  // [parts][Npad][NAp]
+  int parts, NA, NAp, NC, N, Npad, bias, s;
+  float *out, *db;
+};
 bool wgrad_tc_supported(const WgradArgs& w);
 size_t wgrad_tc_partial_floats(const WgradArgs& w, int B);
-void launch_wgrad_tc(const WgradArgs& w, int B, float* partial, float* out, float* db, int* err, cudaStream_t st);
+WgradTcReduceItem launch_wgrad_tc(const WgradArgs& w, int B, float* out, float* db, int* err, cudaStream_t st);
+void launch_wgrad_tc_reduce(const WgradTcReduceItem* items, int n, cudaStream_t st);
 void launch_standardise(const float* x, int B, int C, int L, const float* mean, const float* istd, float* y,
                         cudaStream_t st);
 // loss = (1 / (B Lr)) sum r^2 with r = g (*) (strain - y_hat) valid (Lr = L - K + 1);

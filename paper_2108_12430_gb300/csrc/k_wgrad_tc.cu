@@ -2,24 +2,39 @@
 // operands, FP32 accumulation in TMEM), for the training step's backward.
 //
 // The weight gradient is one contraction over all (item, position) pairs:
-//   dW[a][c][k] = sum_{b, t} A[b][a][t] Bm[b][c][s t + k - p]
+//   dW[a][c][k] = sum_{b, t} A[b][a][t] Bm[b][c][s t + k - 3]
 // (conv: A = the output gradient, Bm = the layer input; transposed conv: A =
 // the layer input, Bm = the output gradient), zero outside [0, LB).  As a
 // GEMM, D[a][n] = sum_t A[a][t] B[n][t] with n = k NC + c and
-// B[n][t] = Bm[c][s t + k - p]: M = the A channels (zero-padded to 128 MMA
-// rows), N = K NC columns, and the reduction runs over positions, which is
-// the dimension the tensor core's K steps walk.
+// B[n][t] = Bm[c][s t + k - 3]: M = the A channels in 128 MMA rows, N = 7 NC
+// columns, and the reduction runs over positions, which is the dimension the
+// tensor core's K steps walk.  A row of ones in A or B gives the bias gradient.
 //
-// Each CTA (512 threads, one per SM) takes chunks of 128 positions of one
-// item in turn.  All its threads stage a chunk: FP32 values are read from
-// global memory once (the A rows and each B channel's raw span), rounded to
-// BF16, and the shifted, strided tap rows of B are built from shared memory,
-// all in the canonical K-major layout (core matrices of 8 rows x 16 bytes);
-// one thread then issues the chunk's eight MMAs into the CTA's TMEM
-// accumulator.  Two stages let the threads fill one while the MMAs read the
-// other.  At the end the
-// accumulator (D, NA x N) goes to the CTA's partial slot, and a second
-// kernel sums the partials in CTA order (deterministic).
+// Bound: neither the tensor core nor DRAM but the way of the operands -- each
+// chunk of positions makes a global round trip, is rounded to BF16 and
+// rearranged, and only then feeds a few MMAs.  So a CTA (one per SM) runs two
+// groups of eight warps, each on its own chunks of 64 positions with its own
+// two shared-memory stages and its own TMEM accumulator: while one group waits
+// for memory or the tensor core, the other stages.  A thread's share of a chunk
+// is fixed: for (row a, 8 positions) it loads 8 values and stores one 16-byte
+// segment; for (channel c, 8 positions) it loads the 16 (stride 1) or 24
+// (stride 2) samples that the seven taps of those positions read and makes all
+// seven tap rows from them in registers, so that no operand passes through
+// shared memory twice.  The next chunk's loads are in flight meanwhile.  Segments
+// of neighbouring positions lie 16 bytes off a multiple of 128 apart (LBO), so
+// that a warp's stores (8 position groups x 4 rows) fall into distinct banks.
+// Rows and columns beyond the operands' are never written: they reach only
+// accumulator rows and columns that are not read.
+//
+// At the end the two accumulators are added and stored column by column (lanes
+// along rows: coalesced) as the CTA's partial; one kernel adds every layer's
+// partials in CTA order (deterministic).
+//
+// Measured (GB300, 32 windows of 21 x 8192, against one group per CTA on chunks
+// of 128, tap rows gathered 2 bytes at a time from shared memory and partials
+// stored row by row): all eight layers 243 -> 144 us (64 x 32 channels 35.6 ->
+// 13.6 us, the first layer 50 -> 30 us), their reductions 55 us in eight launches
+// -> 12 us in one; the BF16 training step 572 -> 398 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -34,13 +49,13 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kWgChunk = 128;    // positions per chunk (eight MMA K steps)
-constexpr int kWgSegs = kWgChunk / 8, kWgLgSegs = 4;  // 16-byte segments of a chunk row
-static_assert((1 << kWgLgSegs) == kWgSegs, "segments per row");
-constexpr int kWgThreads = 512, kWgWarps = kWgThreads / 32;
-constexpr int kWgRowsA = 128;    // MMA M: the A channels, zero-padded
-constexpr int kWgGroup = 6;      // a thread's 16-byte segments of a chunk (all its pass-1 tasks)
-constexpr int kWgMaxCtasPerSm = 1;
+constexpr int kK = 7, kPad = 3;
+constexpr int kChunk = 64, kSegs = kChunk / 8;   // positions per chunk, 16-byte segments per row
+constexpr int kGroups = 2, kGroupWarps = 8, kGroupThreads = 32 * kGroupWarps;
+constexpr int kThreads = kGroups * kGroupThreads;
+constexpr int kRowsA = 128;                      // MMA M
+constexpr int kTasksA = 2;                       // A segments per thread: 64 rows x 8 segments / 256 threads
+constexpr uint32_t kSegA = kRowsA * 16 + 16;     // bytes between neighbouring segments of A (LBO)
 
 struct WgTcParams {
   const float* A;
@@ -49,342 +64,314 @@ struct WgTcParams {
   const float* Bm;
   int64_t bb, bc;  // Bm[b][c][u] at Bm + b bb + c bc + u, u < LB
   int NC, LB;
-  int K, s, p;
-  int N, Npad;     // N = K NC columns n = k NC + c; Npad: the D columns (N, + 1 for bias 1) rounded up to 32
+  int N, Npad;     // N = 7 NC columns n = k NC + c; Npad: the D columns (N, + 1 for bias 1) rounded up to 32
   int bias;        // 1: B row N all ones (D[a][N] = sum_t A[a][t]); 2: A row NA all ones
-  int NAr;         // D rows kept: NA, + 1 for bias 2
-  int span_pad;    // raw B row of a chunk: 63 s + K values, rounded up to 8
-  int a_vec;       // A rows 16-byte aligned at every chunk start
+  int NAr, NAp;    // D rows kept: NA, + 1 for bias 2; rounded up to 8
+  int a_vec, b_vec;  // rows 16-byte aligned at every multiple of 4
   int chunks_per_b, n_chunks;
-  float* partial;  // [gridDim.x][NAr][Npad]
+  float* partial;  // [gridDim.x][Npad][NAp]
   int* err;
 };
 
-// Byte offset of 16-byte segment q (K elements 8q .. 8q + 7) of row r in a
-// K-major tile of R rows: core matrices of 8 rows x 16 bytes, K-adjacent core
-// matrices R / 8 x 128 bytes apart (the descriptor's LBO), row-adjacent ones
-// 128 bytes apart (SBO).
-__device__ __forceinline__ uint32_t seg_off(int r, int q, int R) {
-  return (uint32_t)((((q * (R >> 3)) + (r >> 3)) << 7) + ((r & 7) << 4));
-}
-
-// A chunk cid (item b, positions t0 .. t0 + kWgChunk - 1) is staged by the
-// CTA's warps, each owning the A rows a = w, w + 16, ... and the B channels
-// c = w, w + 16, ... (w its warp index), in two passes that need no
-// synchronisation beyond the warp.  Pass 1 reads global memory once per value:
-// the warp's A rows (task = row, 16-byte segment; 16-byte loads when the row
-// is aligned) and, for each of its B channels c, the raw span u0 .. u0 +
-// span - 1 (u0 = s t0 - p, span = (kWgChunk - 1) s + K) of Bm[c].  Each thread
-// holds its (at most kWgGroup) tasks' 8 values in registers: the loads of
-// chunk i + 1 are issued right after chunk i's values are stored, so that
-// they are in flight while chunk i's tap rows are built and its MMAs issued.
-// The stores round to BF16 into the A tile and raw[c][.].  Pass 2 builds the
-// warp's tap rows B[k NC + c][t] = raw[c][s (t - t0) + k] from shared memory.
-// A task's addresses relative to the chunk are the same for every chunk: each
-// thread works them out once (Pass1Task, tap_task).
-struct Pass1Task {
-  int goff;       // element offset from the chunk's row start (A: row aa + 8 q; B: c bc + j0)
-  int pos;        // position offset: 8 q (A) or j0 (B); -1: no task
-  uint32_t soff;  // A: byte offset in the A tile; B: byte offset in raw
-  bool is_b;
-};
-
-// Rows (or channels) r < n with r = w (mod kWgWarps): how many.
-__host__ __device__ __forceinline__ int owned(int n, int w) { return n > w ? (n - w + kWgWarps - 1) / kWgWarps : 0; }
-
-__device__ __forceinline__ Pass1Task pass1_task(const WgTcParams& p, int w, int task) {
-  Pass1Task t{0, -1, 0u, false};
-  const int span8 = p.span_pad / 8;
-  const int n_a = owned(p.NA, w) * kWgSegs, n_tasks = n_a + owned(p.NC, w) * span8;
-  if (task >= n_tasks) return t;
-  if (task < n_a) {
-    const int row = w + kWgWarps * (task >> kWgLgSegs), q = task & (kWgSegs - 1);
-    t.goff = row * (int)p.aa + 8 * q;
-    t.pos = 8 * q;
-    t.soff = seg_off(row, q, kWgRowsA);
-  } else {
-    const int r = task - n_a, m = r / span8, j0 = (r - m * span8) * 8, c = w + kWgWarps * m;
-    t.goff = c * (int)p.bc + j0;
-    t.pos = j0;
-    t.soff = (uint32_t)(c * p.span_pad + j0) * 2u;
-    t.is_b = true;
-  }
-  return t;
-}
-
-__device__ __forceinline__ void load_chunk(const WgTcParams& p, int cid, const Pass1Task (&tk)[kWgGroup],
-                                           float (&v)[kWgGroup][8]) {
-  const int b = cid / p.chunks_per_b;
-  const int t0 = (cid - b * p.chunks_per_b) * kWgChunk;
-  const int u0 = p.s * t0 - p.p;
-  const float* Ab = p.A + (int64_t)b * p.ab + t0;
-  const float* Bb = p.Bm + (int64_t)b * p.bb + u0;
+// n floats (a multiple of 4) of a row valid in [0, len), from position x0 (a
+// multiple of 4); zeros outside.
+template <int N>
+__device__ __forceinline__ void load_run(const float* row, int x0, int len, bool vec, float* v) {
+  if (vec) {
 #pragma unroll
-  for (int gi = 0; gi < kWgGroup; ++gi) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[gi][e] = 0.f;
-    if (tk[gi].pos < 0) continue;
-    if (!tk[gi].is_b) {
-      const int t = t0 + tk[gi].pos;
-      const float* src = Ab + tk[gi].goff;
-      if (p.a_vec && t + 8 <= p.LA) {
-        const float4 x0 = reinterpret_cast<const float4*>(src)[0], x1 = reinterpret_cast<const float4*>(src)[1];
-        v[gi][0] = x0.x, v[gi][1] = x0.y, v[gi][2] = x0.z, v[gi][3] = x0.w;
-        v[gi][4] = x1.x, v[gi][5] = x1.y, v[gi][6] = x1.z, v[gi][7] = x1.w;
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          if (t + e < p.LA) v[gi][e] = src[e];
+    for (int i = 0; i < N; i += 4) {
+      float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+      const int x = x0 + i;
+      if (x >= 0 && x + 4 <= len) {
+        q = *reinterpret_cast<const float4*>(row + x);
+      } else if (x >= 0) {
+        if (x < len) q.x = row[x];
+        if (x + 1 < len) q.y = row[x + 1];
+        if (x + 2 < len) q.z = row[x + 2];
       }
-    } else {
-      const int u = u0 + tk[gi].pos;
-      const float* src = Bb + tk[gi].goff;
-      if (u >= 0 && u + 8 <= p.LB) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[gi][e] = src[e];
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          if (u + e >= 0 && u + e < p.LB) v[gi][e] = src[e];
-      }
+      v[i] = q.x, v[i + 1] = q.y, v[i + 2] = q.z, v[i + 3] = q.w;
     }
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = (unsigned)(x0 + i) < (unsigned)len ? row[x0 + i] : 0.f;
   }
 }
 
-__device__ __forceinline__ void store_chunk(const Pass1Task (&tk)[kWgGroup], const float (&v)[kWgGroup][8],
-                                            uint8_t* a_smem, uint8_t* raw) {
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+// (high half of a, low half of b)
+__device__ __forceinline__ uint32_t straddle(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x5432); }
+
+// Seven tap rows of 8 positions from the samples w: tap k of position e is
+// w[S e + k + 1].  store(k, segment) receives each.
+template <int S, typename F>
+__device__ __forceinline__ void make_taps(const float* w, F store) {
+  if constexpr (S == 1) {
+    uint32_t even[8];  // (w[2j], w[2j + 1])
 #pragma unroll
-  for (int gi = 0; gi < kWgGroup; ++gi) {
-    if (tk[gi].pos < 0) continue;
-    __nv_bfloat162 h[4];
+    for (int j = 0; j < 8; ++j) even[j] = pack_bf16(w[2 * j], w[2 * j + 1]);
+    uint32_t odd[7];  // (w[2j + 1], w[2j + 2])
 #pragma unroll
-    for (int e = 0; e < 4; ++e) h[e] = __floats2bfloat162_rn(v[gi][2 * e], v[gi][2 * e + 1]);
-    uint8_t* dst = (tk[gi].is_b ? raw : a_smem) + tk[gi].soff;
-    *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(h);
+    for (int j = 0; j < 7; ++j) odd[j] = straddle(even[j], even[j + 1]);
+#pragma unroll
+    for (int k = 0; k < kK; ++k) {
+      const uint32_t* q = (k & 1) ? even + (k + 1) / 2 : odd + k / 2;
+      store(k, make_uint4(q[0], q[1], q[2], q[3]));
+    }
+  } else {
+    // samples of odd index serve the even taps, samples of even index the odd taps
+    uint32_t o[6], e[5], o1[5], e1[4];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) o[j] = pack_bf16(w[4 * j + 1], j < 5 ? w[4 * j + 3] : 0.f);
+#pragma unroll
+    for (int j = 0; j < 5; ++j) e[j] = pack_bf16(w[4 * j + 2], w[4 * j + 4]);
+#pragma unroll
+    for (int j = 0; j < 5; ++j) o1[j] = straddle(o[j], o[j + 1]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) e1[j] = straddle(e[j], e[j + 1]);
+    store(0, make_uint4(o[0], o[1], o[2], o[3]));
+    store(1, make_uint4(e[0], e[1], e[2], e[3]));
+    store(2, make_uint4(o1[0], o1[1], o1[2], o1[3]));
+    store(3, make_uint4(e1[0], e1[1], e1[2], e1[3]));
+    store(4, make_uint4(o[1], o[2], o[3], o[4]));
+    store(5, make_uint4(e[1], e[2], e[3], e[4]));
+    store(6, make_uint4(o1[1], o1[2], o1[3], o1[4]));
   }
 }
 
-// Pass 2 task (tap row n = k NC + c of one of the warp's channels c, segment
-// q): source element offset in raw (low 16 bits) and offset in the B tile in
-// 16-byte units (high 16 bits); ~0u: no task.
-constexpr int kWgTaps = 12;
-__device__ __forceinline__ uint32_t tap_task(const WgTcParams& p, int w, int task) {
-  const int per_c = p.K * kWgSegs;
-  if (task >= owned(p.NC, w) * per_c) return ~0u;
-  const int m = task / per_c, r = task - m * per_c, k = r >> kWgLgSegs, q = r & (kWgSegs - 1);
-  const int c = w + kWgWarps * m, n = k * p.NC + c;
-  return (uint32_t)(c * p.span_pad + p.s * 8 * q + k) | ((seg_off(n, q, p.Npad) >> 4) << 16);
-}
-
-__device__ __forceinline__ void build_taps(const WgTcParams& p, const uint32_t (&tt)[kWgTaps], uint8_t* b_smem,
-                                           const __nv_bfloat16* raw) {
-#pragma unroll
-  for (int it = 0; it < kWgTaps; ++it) {
-    if (tt[it] == ~0u) continue;
-    const __nv_bfloat16* src = raw + (tt[it] & 0xffffu);
-    __align__(16) __nv_bfloat16 h[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) h[e] = src[p.s * e];
-    *reinterpret_cast<uint4*>(b_smem + ((tt[it] >> 16) << 4)) = *reinterpret_cast<const uint4*>(h);
-  }
-}
-
-__global__ void __launch_bounds__(kWgThreads, kWgMaxCtasPerSm) wgrad_tc_kernel(const WgTcParams p) {
+template <int S>
+__global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_constant__ WgTcParams p) {
+  // B segments per thread: 8 per channel; stride 1 (the network's first layer)
+  // takes up to 64 channels, stride 2 up to 32
+  constexpr int kTasksB = S == 1 ? 2 : 1, kW = S == 1 ? 16 : 24;
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  const uint32_t base = smem_u32(smem);
-  const uint32_t a_bytes = kWgRowsA * kWgChunk * 2, b_bytes = (uint32_t)p.Npad * kWgChunk * 2;
-  const uint32_t stage_bytes = a_bytes + b_bytes;
-  // [0..1] stage free (its MMAs done), [2] all MMAs done, [3..4] stage staged (one arrival per warp)
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * stage_bytes);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 5);
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+  const uint32_t seg_b = (uint32_t)p.Npad * 16u + 16u;
+  const uint32_t a_bytes = kSegs * kSegA, stage_bytes = (a_bytes + kSegs * seg_b + 127u) & ~127u;
+  // per group: [0..1] stage free (its MMAs done), [2..3] stage staged (one arrival per warp), [4] all MMAs done
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * kGroups * stage_bytes);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 5 * kGroups);
   uint32_t* tslot = (uint32_t*)(abort_flag + 1);
-  __nv_bfloat16* raw = reinterpret_cast<__nv_bfloat16*>(smem + 2 * stage_bytes + 64);  // [NC][span_pad]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int grp = tid / kGroupThreads, gt = tid - grp * kGroupThreads;
+  uint8_t* stages = smem + grp * 2 * stage_bytes;
+  auto bar = [&](int g, int i) { return smem_u32(&bars[5 * g + i]); };
 
-  // both stages start at zero: the A rows >= NA and B rows >= N are never
-  // written and contribute zeros
-  {
-    uint4* z = reinterpret_cast<uint4*>(smem);
-    for (uint32_t i = tid; i < 2 * stage_bytes / 16; i += kWgThreads) z[i] = make_uint4(0u, 0u, 0u, 0u);
-  }
   if (tid == 0) {
-    for (int i = 0; i < 3; ++i) mbar_init(smem_u32(&bars[i]), 1);
-    for (int i = 3; i < 5; ++i) mbar_init(smem_u32(&bars[i]), kWgWarps);
+    for (int g = 0; g < kGroups; ++g) {
+      for (int i = 0; i < 5; ++i) mbar_init(bar(g, i), (i == 2 || i == 3) ? kGroupWarps : 1);
+    }
     *abort_flag = 0u;
     fence_barrier_init();
   }
-  __syncthreads();
   if (p.bias) {
-    // the bias row of ones (BF16 1.0) in both stages: staging never writes it
+    // the row of ones (BF16 1.0) in every stage: staging never writes it
     const uint4 ones = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
-    if (tid < 2 * kWgSegs) {
-      const int st = tid >> kWgLgSegs, q = tid & (kWgSegs - 1);
-      uint8_t* tile = smem + st * stage_bytes + (p.bias == 1 ? a_bytes : 0u);
-      *reinterpret_cast<uint4*>(tile + (p.bias == 1 ? seg_off(p.N, q, p.Npad) : seg_off(p.NA, q, kWgRowsA))) = ones;
+    if (gt < 2 * kSegs) {
+      const int r = p.bias == 1 ? p.N : p.NA, q = gt & (kSegs - 1);
+      uint8_t* tile = stages + (gt / kSegs) * stage_bytes + (p.bias == 1 ? a_bytes + q * seg_b : q * kSegA);
+      *reinterpret_cast<uint4*>(tile + (r >> 3) * 128 + (r & 7) * 16) = ones;
     }
   }
   fence_proxy_async_smem();
-  const uint32_t tcols = p.Npad <= 128 ? 128u : 256u;
-  if (warp == 0) tmem_alloc(smem_u32(tslot), tcols);
+  const uint32_t acc_cols = p.Npad <= 128 ? 128u : 256u;
+  if (warp == 0) tmem_alloc(smem_u32(tslot), kGroups * acc_cols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = *tslot + grp * acc_cols;
   // D = F32, A = B = BF16, both K-major, N >> 3 at bit 17, M >> 4 at bit 24
   const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.Npad >> 3) << 17) |
-                         ((uint32_t)(kWgRowsA >> 4) << 24);
-  const uint32_t lbo_a = (kWgRowsA / 8) * 128, lbo_b = (uint32_t)(p.Npad / 8) * 128;
+                         ((uint32_t)(kRowsA >> 4) << 24);
 
+  // this thread's tasks: (row, segment) pairs, segments fastest
+  const float* a_row[kTasksA];
+  uint32_t a_dst[kTasksA];
+  bool a_on[kTasksA];
+  const int q = gt & (kSegs - 1);  // the same segment for all of them
+#pragma unroll
+  for (int i = 0; i < kTasksA; ++i) {
+    const int a = (gt >> 3) + i * (kGroupThreads / kSegs);
+    a_on[i] = a < p.NA;
+    a_row[i] = p.A + (int64_t)(a_on[i] ? a : 0) * p.aa;
+    a_dst[i] = (uint32_t)(q * kSegA + (a >> 3) * 128 + (a & 7) * 16);
+  }
+  const float* b_row[kTasksB];
+  int b_c[kTasksB];
+#pragma unroll
+  for (int i = 0; i < kTasksB; ++i) {
+    const int c = (gt >> 3) + i * (kGroupThreads / kSegs);
+    b_c[i] = c < p.NC ? c : -1;
+    b_row[i] = p.Bm + (int64_t)(c < p.NC ? c : 0) * p.bc;
+  }
+  float av[kTasksA][8], bv[kTasksB][kW];
+  auto load = [&](int chunk) {
+    const int b = chunk / p.chunks_per_b, t = (chunk - b * p.chunks_per_b) * kChunk + 8 * q;
+#pragma unroll
+    for (int i = 0; i < kTasksA; ++i)
+      if (a_on[i]) load_run<8>(a_row[i] + (int64_t)b * p.ab, t, p.LA, p.a_vec, av[i]);
+#pragma unroll
+    for (int i = 0; i < kTasksB; ++i)
+      if (b_c[i] >= 0) load_run<kW>(b_row[i] + (int64_t)b * p.bb, S * t - kPad - 1, p.LB, p.b_vec, bv[i]);
+  };
+
+  griddep_wait();  // operands come from the previous kernels
   int i = 0;
-  Pass1Task tk[kWgGroup];
-#pragma unroll
-  for (int gi = 0; gi < kWgGroup; ++gi) tk[gi] = pass1_task(p, warp, lane + 32 * gi);
-  uint32_t tt[kWgTaps];
-#pragma unroll
-  for (int it = 0; it < kWgTaps; ++it) tt[it] = tap_task(p, warp, lane + 32 * it);
-  float v[kWgGroup][8];
-  if ((int)blockIdx.x < p.n_chunks) load_chunk(p, blockIdx.x, tk, v);
-  for (int cid = blockIdx.x; cid < p.n_chunks; cid += gridDim.x, ++i) {
+  const int first = blockIdx.x * kGroups + grp, step = gridDim.x * kGroups;
+  if (first < p.n_chunks) load(first);
+  for (int chunk = first; chunk < p.n_chunks; chunk += step, ++i) {
     const int st = i & 1;
     // the stage's previous MMAs (chunk i - 2) have read it
     bool ok = true;
-    if (i >= 2 && lane == 0) ok = mbar_wait(smem_u32(&bars[st]), (uint32_t)((i - 2) >> 1) & 1u, abort_flag, p.err, 1);
+    if (i >= 2 && lane == 0) ok = mbar_wait(bar(grp, st), (uint32_t)((i - 2) >> 1) & 1u, abort_flag, p.err, 1);
     if (!__shfl_sync(0xffffffffu, ok ? 1 : 0, 0)) break;
-    uint8_t* a_s = smem + st * stage_bytes;
-    store_chunk(tk, v, a_s, reinterpret_cast<uint8_t*>(raw));
-    if (cid + (int)gridDim.x < p.n_chunks) load_chunk(p, cid + gridDim.x, tk, v);
-    __syncwarp();  // the warp's raw rows are complete
-    build_taps(p, tt, a_s + a_bytes, raw);
+    uint8_t* a_s = stages + st * stage_bytes;
+    uint8_t* b_s = a_s + a_bytes + q * seg_b;
+#pragma unroll
+    for (int x = 0; x < kTasksA; ++x)
+      if (a_on[x])
+        *reinterpret_cast<uint4*>(a_s + a_dst[x]) =
+            make_uint4(pack_bf16(av[x][0], av[x][1]), pack_bf16(av[x][2], av[x][3]), pack_bf16(av[x][4], av[x][5]),
+                       pack_bf16(av[x][6], av[x][7]));
+#pragma unroll
+    for (int x = 0; x < kTasksB; ++x)
+      if (b_c[x] >= 0)
+        make_taps<S>(bv[x], [&](int k, uint4 seg) {
+          const int n = k * p.NC + b_c[x];
+          *reinterpret_cast<uint4*>(b_s + (n >> 3) * 128 + (n & 7) * 16) = seg;
+        });
+    if (chunk + step < p.n_chunks) load(chunk + step);
     fence_proxy_async_smem();  // the stores above are read by the tensor core (async proxy)
     __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&bars[3 + st]));
-    if (tid == 0) {
-      // every warp has staged its part of the chunk
-      ok = mbar_wait(smem_u32(&bars[3 + st]), (uint32_t)(i >> 1) & 1u, abort_flag, p.err, 4);
+    if (lane == 0) mbar_arrive(bar(grp, 2 + st));
+    if (gt == 0) {
+      // every warp of the group has staged its part of the chunk
+      ok = mbar_wait(bar(grp, 2 + st), (uint32_t)(i >> 1) & 1u, abort_flag, p.err, 4);
       if (ok) {
         tc_fence_after();
-        const uint32_t a0 = base + st * stage_bytes, b0 = a0 + a_bytes;
+        const uint32_t a0 = smem_u32(a_s), b0 = a0 + a_bytes;
 #pragma unroll
-        for (int j = 0; j < kWgChunk / 16; ++j)
-          mma_f16(tmem, make_desc(a0 + 2 * j * lbo_a, lbo_a, 128), make_desc(b0 + 2 * j * lbo_b, lbo_b, 128), idesc,
+        for (int j = 0; j < kChunk / 16; ++j)
+          mma_f16(tmem, make_desc(a0 + 2 * j * kSegA, kSegA, 128), make_desc(b0 + 2 * j * seg_b, seg_b, 128), idesc,
                   (i > 0 || j > 0) ? 1u : 0u);
-        mma_commit(smem_u32(&bars[st]));
+        mma_commit(bar(grp, st));
       }
     }
     if (!__shfl_sync(0xffffffffu, ok ? 1 : 0, 0)) break;
   }
   __syncthreads();
-  // every MMA of this CTA has completed before the accumulator is read
-  if (tid == 0) mma_commit(smem_u32(&bars[2]));
-  mbar_wait_landed(smem_u32(&bars[2]), 0u, p.err, 2);
+  // every MMA of this CTA has completed before the accumulators are read
+  if (gt == 0) mma_commit(bar(grp, 4));
+  for (int g = 0; g < kGroups; ++g) mbar_wait_landed(bar(g, 4), 0u, p.err, 2);
   tc_fence_after();
-  if (warp < 4) {
-    const int r = warp * 32 + lane;  // TMEM lane = MMA row = A channel
-    float* dst = p.partial + ((int64_t)blockIdx.x * p.NAr + r) * p.Npad;
-    for (int c0 = 0; c0 < p.Npad; c0 += 32) {
-      float v[32];
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+  // warp w reads TMEM lanes 32 (w % 4) .. and every fourth block of 32 columns
+  const int r = (warp & 3) * 32 + lane;  // TMEM lane = MMA row = A channel
+  if ((warp & 3) * 32 < p.NAr) {
+    float* dst = p.partial + (int64_t)blockIdx.x * p.Npad * p.NAp + r;
+    const uint32_t t0 = *tslot + ((uint32_t)((warp & 3) * 32) << 16);
+    const bool used0 = blockIdx.x * kGroups < p.n_chunks, used1 = blockIdx.x * kGroups + 1 < p.n_chunks;
+    for (int c0 = 32 * (warp >> 2); c0 < p.Npad; c0 += 32 * (kThreads / 128)) {
+      float v[32], u[32];
+      tmem_ld32(t0 + (uint32_t)c0, v);
+      tmem_ld32(t0 + acc_cols + (uint32_t)c0, u);
       if (r < p.NAr) {
 #pragma unroll
-        for (int q = 0; q < 32; ++q) dst[c0 + q] = i > 0 ? v[q] : 0.f;
+        for (int x = 0; x < 32; ++x)
+          dst[(int64_t)(c0 + x) * p.NAp] = (used0 ? v[x] : 0.f) + (used1 ? u[x] : 0.f);
       }
     }
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, tcols);
+  if (warp == 0) tmem_dealloc(*tslot, kGroups * acc_cols);
 }
 
-// out[a][c][k] = sum over CTAs g of partial[g][a][k NC + c].  A block takes
-// 32 consecutive (a, n) columns of the partials; warp w sums g = w, w + 8, ...
-// in order (lanes on consecutive n: coalesced), then the eight warp sums are
-// added in warp order, so the result does not depend on the schedule.  The
-// bias gradient: bias 1, db[a] = the sum of column N; bias 2, db[c] = the
-// sum of row NA's columns k NC + c for k = p .. p + s - 1 (the taps that put
-// every output position u = s t + k - p of channel c in exactly one (t, k)).
-constexpr int kWgRedWarps = 8;
-struct WgRedParams {
-  const float* partial;
-  int G, NA, NAr, NC, K, N, Npad, bias, s, p;
-  float* out;
-  float* db;
+// Sums of every layer's partials, in CTA order: a block takes 32 consecutive
+// values of one layer's [Npad][NAp] (blockIdx.y: the layer), warp w the CTAs w,
+// w + 8, ..., and the eight sums are added in warp order.  The bias gradient:
+// bias 1, db[a] = column N; bias 2, db[c] = the sum of row NA's columns k NC +
+// c over taps 3 .. 3 + s - 1 (every output position u = s t + k - 3 of channel c
+// is in exactly one such (t, k)).
+constexpr int kRedWarps = 8;
+struct ReduceList {
+  WgradTcReduceItem it[kWgradReduceMax];
 };
-__global__ void __launch_bounds__(32 * kWgRedWarps) wgrad_tc_reduce_kernel(const WgRedParams q) {
-  __shared__ float red[kWgRedWarps][32];
+__global__ void __launch_bounds__(32 * kRedWarps) wgrad_tc_reduce_kernel(const __grid_constant__ ReduceList l) {
+  __shared__ float red[kRedWarps][32];
+  const WgradTcReduceItem& q = l.it[blockIdx.y];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t e = (int64_t)blockIdx.x * 32 + lane;  // index into [NAr][Npad]
-  const int64_t stride = (int64_t)q.NAr * q.Npad;
-  const int a = (int)(e / q.Npad), n = (int)(e - (int64_t)a * q.Npad);
-  // the partial columns this lane adds (cnt of them, NC apart)
+  const int e = blockIdx.x * 32 + lane, stride = q.Npad * q.NAp;  // index into [Npad][NAp]
+  if ((int)blockIdx.x * 32 >= stride) return;
+  const int n = e / q.NAp, a = e - n * q.NAp;
+  // the values this lane adds (cnt of them, NC columns apart)
   int cnt = 0;
   if (e < stride) {
     if (a < q.NA)
       cnt = (n < q.N || (q.bias == 1 && n == q.N)) ? 1 : 0;
-    else if (n < q.N && n / q.NC == q.p)
+    else if (q.bias == 2 && a == q.NA && n < q.N && n / q.NC == kPad)
       cnt = q.s;
   }
   float acc = 0.f;
   for (int j = 0; j < cnt; ++j) {
     // four CTAs' partials in flight per step
-    const float* src = q.partial + e + j * q.NC;
+    const float* src = q.partial + e + j * q.NC * q.NAp;
     int g = warp;
-    for (; g + 3 * kWgRedWarps < q.G; g += 4 * kWgRedWarps) {
-      const float v0 = src[(int64_t)g * stride], v1 = src[(int64_t)(g + kWgRedWarps) * stride];
-      const float v2 = src[(int64_t)(g + 2 * kWgRedWarps) * stride], v3 = src[(int64_t)(g + 3 * kWgRedWarps) * stride];
+    for (; g + 3 * kRedWarps < q.parts; g += 4 * kRedWarps) {
+      const float v0 = src[(int64_t)g * stride], v1 = src[(int64_t)(g + kRedWarps) * stride];
+      const float v2 = src[(int64_t)(g + 2 * kRedWarps) * stride], v3 = src[(int64_t)(g + 3 * kRedWarps) * stride];
       acc += v0;
       acc += v1;
       acc += v2;
       acc += v3;
     }
-    for (; g < q.G; g += kWgRedWarps) acc += src[(int64_t)g * stride];
+    for (; g < q.parts; g += kRedWarps) acc += src[(int64_t)g * stride];
   }
   red[warp][lane] = acc;
   __syncthreads();
   if (warp == 0 && cnt > 0) {
     float t = 0.f;
-    for (int w = 0; w < kWgRedWarps; ++w) t += red[w][lane];
+    for (int w = 0; w < kRedWarps; ++w) t += red[w][lane];
     if (a < q.NA && n < q.N) {
       const int k = n / q.NC, c = n - k * q.NC;
-      q.out[((int64_t)a * q.NC + c) * q.K + k] = t;
+      q.out[((int64_t)a * q.NC + c) * kK + k] = t;
     } else if (a < q.NA) {
       q.db[a] = t;
     } else {
-      q.db[n - q.p * q.NC] = t;
+      q.db[n - kPad * q.NC] = t;
     }
   }
 }
 
 int wgrad_tc_grid(const WgradArgs& w, int B) {
-  const int chunks = B * ((w.LA + kWgChunk - 1) / kWgChunk);
-  return std::max(1, std::min(chunks, kWgMaxCtasPerSm * current_sm_count()));
+  const int chunks = B * ((w.LA + kChunk - 1) / kChunk);
+  return std::max(1, std::min((chunks + kGroups - 1) / kGroups, current_sm_count()));
+}
+// D's columns (N, + 1 for the ones row of bias 1) rounded up to 32, and rows
+// (NA, + 1 for bias 2) rounded up to 8.
+int wg_npad(const WgradArgs& w) { return (kK * w.NC + (w.bias == 1 ? 1 : 0) + 31) / 32 * 32; }
+int wg_rows(const WgradArgs& w) { return w.NA + (w.bias == 2 ? 1 : 0); }
+size_t wg_smem(int npad) {
+  const size_t stage = (kSegs * kSegA + kSegs * ((size_t)npad * 16 + 16) + 127) / 128 * 128;
+  return 128 + 2 * kGroups * stage + 5 * kGroups * 8 + 16;
 }
 
-}  // namespace
-
-namespace {
-// D's columns (N, + 1 for the ones row of bias 1) rounded up to 32, and rows
-// (NA, + 1 for bias 2).
-int wg_npad(const WgradArgs& w) { return (w.K * w.NC + (w.bias == 1 ? 1 : 0) + 31) / 32 * 32; }
-int wg_rows(const WgradArgs& w) { return w.NA + (w.bias == 2 ? 1 : 0); }
 }  // namespace
 
 bool wgrad_tc_supported(const WgradArgs& w) {
-  const int span_pad = ((kWgChunk - 1) * w.s + w.K + 7) / 8 * 8;
-  // bias 2 sums taps p .. p + s - 1 of every t < LA: each output position
-  // u < LB exactly once when LB = s LA
-  const bool bias_ok = w.bias == 0 || w.bias == 1 || (w.bias == 2 && w.LB == w.s * w.LA && w.p + w.s <= w.K);
-  return tc_supported() && bias_ok && w.NA >= 1 && wg_rows(w) <= kWgRowsA && w.NC >= 1 && wg_npad(w) <= 256 &&
-         owned(w.NA, 0) * kWgSegs + owned(w.NC, 0) * (span_pad / 8) <= 32 * kWgGroup &&
-         owned(w.NC, 0) * w.K * kWgSegs <= 32 * kWgTaps && w.NC * span_pad < 65536 &&
-         (int64_t)w.NA * w.aa < (1LL << 31) && (int64_t)w.NC * w.bc < (1LL << 31);
+  // bias 2 sums taps 3 .. 3 + s - 1 of every t < LA: each output position u < LB exactly once when LB = s LA
+  const bool bias_ok = w.bias == 0 || w.bias == 1 || (w.bias == 2 && w.LB == w.s * w.LA);
+  const int channels = (w.s == 1 ? 2 : 1) * kGroupThreads / kSegs;
+  return tc_supported() && bias_ok && w.K == kK && w.p == kPad && (w.s == 1 || w.s == 2) && w.NA >= 1 &&
+         w.NA <= kTasksA * kGroupThreads / kSegs && w.NC >= 1 && w.NC <= channels && wg_npad(w) <= 256;
 }
 
 size_t wgrad_tc_partial_floats(const WgradArgs& w, int B) {
-  return (size_t)wgrad_tc_grid(w, B) * wg_rows(w) * wg_npad(w);
+  return (size_t)wgrad_tc_grid(w, B) * wg_npad(w) * ((wg_rows(w) + 7) / 8 * 8);
 }
 
-void launch_wgrad_tc(const WgradArgs& w, int B, float* partial, float* out, float* db, int* err, cudaStream_t st) {
+WgradTcReduceItem launch_wgrad_tc(const WgradArgs& w, int B, float* out, float* db, int* err, cudaStream_t st) {
   GW_CHECK_ARG(wgrad_tc_supported(w), "layer shape outside the tensor-core weight-gradient kernel");
   GW_CHECK_ARG(!w.bias || db, "bias gradient requested without an output");
   WgTcParams p{};
@@ -398,33 +385,44 @@ void launch_wgrad_tc(const WgradArgs& w, int B, float* partial, float* out, floa
   p.bc = w.bc;
   p.NC = w.NC;
   p.LB = w.LB;
-  p.K = w.K;
-  p.s = w.s;
-  p.p = w.p;
-  p.N = w.K * w.NC;
+  p.N = kK * w.NC;
   p.Npad = wg_npad(w);
   p.bias = w.bias;
   p.NAr = wg_rows(w);
-  p.span_pad = ((kWgChunk - 1) * w.s + w.K + 7) / 8 * 8;
-  p.a_vec = (w.aa % 4 == 0 && w.ab % 4 == 0 && ((uintptr_t)w.A & 15) == 0) ? 1 : 0;
-  p.chunks_per_b = (w.LA + kWgChunk - 1) / kWgChunk;
+  p.NAp = (p.NAr + 7) / 8 * 8;
+  p.a_vec = w.aa % 4 == 0 && w.ab % 4 == 0 && ((uintptr_t)w.A & 15) == 0;
+  p.b_vec = w.bc % 4 == 0 && w.bb % 4 == 0 && ((uintptr_t)w.Bm & 15) == 0;
+  p.chunks_per_b = (w.LA + kChunk - 1) / kChunk;
   p.n_chunks = B * p.chunks_per_b;
-  p.partial = partial;
+  p.partial = w.partial;
   p.err = err;
   const int grid = wgrad_tc_grid(w, B);
-  // at least 80 KB of shared memory per CTA, so that at most two CTAs share an
-  // SM and their TMEM allocations (up to 256 columns each) always fit
-  const size_t raw_bytes = (size_t)w.NC * p.span_pad * 2;
-  const size_t smem = std::max<size_t>(kWgMaxCtasPerSm == 2 ? 80 * 1024 : 0,
-                                       1024 + 2 * (size_t)(kWgRowsA + p.Npad) * kWgChunk * 2 + 64 + raw_bytes);
-  GW_CHECK_ARG(smem <= 227 * 1024, "weight-gradient tile exceeds shared memory");
+  auto kernel = w.s == 1 ? wgrad_tc_kernel<1> : wgrad_tc_kernel<2>;
   // the limit is set once per device, to the most any layer may ask for
-  set_smem_limit_once(wgrad_tc_kernel, 227 * 1024);
-  wgrad_tc_kernel<<<grid, kWgThreads, smem, st>>>(p);
-  GW_LAUNCH_CHECK();
-  WgRedParams q{partial, grid, w.NA, p.NAr, w.NC, w.K, p.N, p.Npad, w.bias, w.s, w.p, out, db};
-  const int64_t cols = (int64_t)p.NAr * p.Npad;
-  wgrad_tc_reduce_kernel<<<(unsigned)((cols + 31) / 32), 32 * kWgRedWarps, 0, st>>>(q);
+  set_smem_limit_once(kernel, 227 * 1024);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = wg_smem(p.Npad);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  GW_CUDA(cudaLaunchKernelEx(&cfg, kernel, p));
+  return {w.partial, grid, w.NA, p.NAp, w.NC, p.N, p.Npad, w.bias, w.s, out, db};
+}
+
+void launch_wgrad_tc_reduce(const WgradTcReduceItem* items, int n, cudaStream_t st) {
+  GW_CHECK_ARG(n >= 1 && n <= kWgradReduceMax, "reduction list size");
+  ReduceList l{};
+  int mx = 1;
+  for (int i = 0; i < n; ++i) {
+    l.it[i] = items[i];
+    mx = std::max(mx, items[i].Npad * items[i].NAp);
+  }
+  wgrad_tc_reduce_kernel<<<dim3((mx + 31) / 32, n), 32 * kRedWarps, 0, st>>>(l);
   GW_LAUNCH_CHECK();
 }
 

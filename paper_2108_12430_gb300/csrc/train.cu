@@ -444,7 +444,9 @@ int gw_trainer_backward(gw_trainer_t t, const float* dy_hat, float* dparams, voi
   const float* g = dy_hat;  // gradient w.r.t. the current layer's (pre-activation) output
   int64_t gb = t->L, gn = t->L;
   int cur = 0;
-  std::vector<WgradReduceItem> reduce;  // FP32 weight gradients: added up by one launch at the end
+  // weight gradients' partials: added up by one launch at the end
+  std::vector<WgradReduceItem> reduce;
+  std::vector<WgradTcReduceItem> reduce_tc;
   TcOut gnext{};  // tc_data: the next data gradient's input, blocked by the previous one
   for (int l = nl - 1; l >= 0; --l) {
     const TrainLayer& T = t->layers[l];
@@ -467,7 +469,7 @@ int gw_trainer_backward(gw_trainer_t t, const float* dy_hat, float* dparams, voi
     w.partial = t->partial[l];
     if (t->wgrad_tc && wgrad_tc_supported(w)) {
       Prof p(l < 8 ? kWgradTcNames[l] : "train.wgrad_tc", st);
-      launch_wgrad_tc(w, B, w.partial, t->dWf[l], t->dbf[l], t->err, st);
+      reduce_tc.push_back(launch_wgrad_tc(w, B, t->dWf[l], t->dbf[l], t->err, st));
     } else {
       Prof p(l < 8 ? kWgradNames[l] : "train.wgrad", st);
       reduce.push_back(launch_wgrad_f32(w, B, t->dWf[l], t->dbf[l], st));
@@ -555,6 +557,10 @@ int gw_trainer_backward(gw_trainer_t t, const float* dy_hat, float* dparams, voi
   for (size_t i = 0; i < reduce.size(); i += kWgradReduceMax) {
     Prof p("train.wgrad_reduce", st);
     launch_wgrad_reduce(reduce.data() + i, (int)std::min<size_t>(kWgradReduceMax, reduce.size() - i), st);
+  }
+  for (size_t i = 0; i < reduce_tc.size(); i += kWgradReduceMax) {
+    Prof p("train.wgrad_reduce", st);
+    launch_wgrad_tc_reduce(reduce_tc.data() + i, (int)std::min<size_t>(kWgradReduceMax, reduce_tc.size() - i), st);
   }
   {
     // every layer's chain rule from the folded to the raw parameters, one launch
