@@ -26,7 +26,7 @@
 //
 // Kernel.  Persistent and warp-specialised: warps 0 and 10 stage input tiles
 // by bulk TMA into a ring of up to 6 stages (alternate tiles; zero rows for the
-// padding at the edges), warp 1 issues the MMAs from one thread into a
+// padding at the edges), warp 1 issues the MMAs (one elected lane) into a
 // double-buffered TMEM accumulator, warps 2-9 drain TMEM with tcgen05.ld, add
 // bias (and a residual), apply the activation and store the consumer's layout.
 // Weights stay resident in shared memory when they fit, else stream per tile
@@ -77,6 +77,19 @@ constexpr int kErrWaitA = 1, kErrWaitW = 2, kErrWaitAcc = 4, kErrWaitEmpty = 8, 
 constexpr int kZeroRows = 2048;
 __device__ __align__(128) uint4 g_zero_rows[kZeroRows];
 
+// n / d for n < 2^31 by a multiplication: a runtime division takes about 150
+// cycles of the single thread that runs it, and every role made several per
+// tile and weight stage.
+struct FastDiv {
+  uint32_t mul, shift;
+};
+FastDiv fast_div(uint32_t d) {
+  uint32_t l = 0;
+  while ((1ull << l) < d) ++l;
+  return {(uint32_t)(((1ull << 32) * ((1ull << l) - d)) / d + 1), l};
+}
+__device__ __forceinline__ uint32_t div_by(uint32_t n, const FastDiv& f) { return (__umulhi(n, f.mul) + n) >> f.shift; }
+
 struct TcParams {
   const char* in;
   int64_t in_off0, in_b, in_boff, in_g, in_p;  // bytes (boff in 16-byte rows)
@@ -88,7 +101,13 @@ struct TcParams {
   int na;  // input stages in the A ring (2..kMaxA)
   // output-channel split: a tile is (M tile, column slice); each slice has
   // ncol = npad / nsplit columns (used when a layer has fewer tiles than SMs)
-  int nsplit, ncol;
+  int nsplit, ncol, nsplit_log;
+  FastDiv div_tpi;  // by tiles_per_item
+  // one M tile per item: every tile's padding rows are the same rows of the
+  // stage, zeroed once per CTA instead of copied with every tile (a copy costs
+  // its warp about 60 cycles whatever its size, and both edges treble them: the
+  // 256 -> 256 channel layer on 256 items 44.9 us, 40.5 us so)
+  int prezero;
   // streamed weight stages: bytes per K-step in a stage (step_bytes, or with
   // wcompact = 1 only the slice's rows, packed [K-half][ncol rows] per step),
   // and the producer warps that fill them (1, or 2 with an even nst)
@@ -150,10 +169,11 @@ __device__ __forceinline__ bool epi_bar_and(bool ok) {
 // whose stride is a multiple of half the tiles per item met an edge tile on
 // every other step.
 __device__ __forceinline__ void tile_coords(const TcParams& p, int t, int& b, int& m0, int& sl) {
-  const int tm = t / p.nsplit;
-  sl = t - tm * p.nsplit;
-  b = tm / p.tiles_per_item;
-  int j = tm - b * p.tiles_per_item + b % p.tiles_per_item;
+  const int tm = t >> p.nsplit_log;
+  sl = t & (p.nsplit - 1);
+  b = (int)div_by((uint32_t)tm, p.div_tpi);
+  const int turn = b - (int)div_by((uint32_t)b, p.div_tpi) * p.tiles_per_item;
+  int j = tm - b * p.tiles_per_item + turn;
   if (j >= p.tiles_per_item) j -= p.tiles_per_item;
   m0 = j * 128 * p.MT;
 }
@@ -238,6 +258,12 @@ __global__ void __launch_bounds__(kThreads, kMaxCtasPerSm) conv_tc_kernel(const 
     s_poff[i] = (int64_t)g * p.in_g + (int64_t)phi * p.in_p;
     s_plen[i] = (p.in_L - phi + p.in_P - 1) / p.in_P;
   }
+  if (p.prezero) {
+    uint4* z = reinterpret_cast<uint4*>(smem);
+    const int n16 = na * p.a_bytes / 16;
+    for (int i = tid; i < n16; i += kThreads) z[i] = make_uint4(0u, 0u, 0u, 0u);
+    fence_proxy_async_smem();
+  }
   for (int i = tid; i < p.npad; i += kThreads) {
     s_bias[i] = i < p.cout ? p.bias[i] : 0.f;
     s_scale[i] = (p.wscale && i < p.cout) ? p.wscale[i] : 1.f;
@@ -276,9 +302,10 @@ __global__ void __launch_bounds__(kThreads, kMaxCtasPerSm) conv_tc_kernel(const 
     }
     griddep_wait();
     int i = 0;
-    int s = 0, k = 0;  // ring stage and its use count, advanced without divisions
+    int s = 0, k = 0;     // ring stage and its use count, advanced without divisions
+    int wst = 0, wk = 0;  // the same of the weight ring
     for (int t = blockIdx.x; t < p.n_tiles; t += gridDim.x, ++i, k += (++s == na), s = s == na ? 0 : s) {
-      const bool do_a = i % nprod == pw, do_w = !p.resident && pw < p.wprod;
+      const bool do_a = nprod == 1 ? pw == 0 : (i & 1) == pw, do_w = !p.resident && pw < p.wprod;
       if (!do_a && !do_w) continue;
       if (p.stall_test && blockIdx.x == 0 && i == 0) continue;  // no arrival and no copy: nothing in flight
       int b, m0, sl;
@@ -290,7 +317,23 @@ __global__ void __launch_bounds__(kThreads, kMaxCtasPerSm) conv_tc_kernel(const 
         const char* src0 = p.item_ptr
                                ? p.item_ptr[b] + (int64_t)base * 16
                                : p.in + p.in_off0 + (int64_t)b * p.in_b + ((int64_t)base + (int64_t)b * p.in_boff) * 16;
-        if (base >= 0 && base + p.rows <= p.min_plen) {
+        if (p.prezero) {
+          // the item's own rows of every plane; the padding rows stay zero
+          int n = 0;
+          for (int plane = lane; plane < planes; plane += 32) {
+            const int r0 = min(p.rows, max(0, -base));
+            n += max(r0, min(p.rows, s_plen[plane] - base)) - r0;
+          }
+          n = __reduce_add_sync(0xffffffffu, n);
+          if (lane == 0) mbar_expect_tx(bar(a_full + s), (uint32_t)n * 16u);
+          __syncwarp();
+          for (int plane = lane; plane < planes; plane += 32) {
+            const int r0 = min(p.rows, max(0, -base)), r1 = max(r0, min(p.rows, s_plen[plane] - base));
+            if (r1 > r0)
+              bulk_g2s(sAs + (uint32_t)(plane * p.rows + r0) * 16u, src0 + s_poff[plane] + (int64_t)r0 * 16,
+                       (uint32_t)(r1 - r0) * 16u, bar(a_full + s));
+          }
+        } else if (base >= 0 && base + p.rows <= p.min_plen) {
           // interior tile: every plane is one full run of rows
           if (lane == 0) mbar_expect_tx(bar(a_full + s), (uint32_t)(planes * p.rows) * 16u);
           __syncwarp();
@@ -317,10 +360,10 @@ __global__ void __launch_bounds__(kThreads, kMaxCtasPerSm) conv_tc_kernel(const 
       }
       if (lane == 0) {
         if (do_w) {
-          for (int c = 0; c < n_chunks; ++c) {
-            const int gc = i * n_chunks + c, st = gc % p.nst, use = gc / p.nst;
-            if (gc % p.wprod != pw) continue;
-            if (use >= 1 && !mbar_wait(bar(w_empty + st), (uint32_t)(use - 1) & 1u, abort_flag, p.err, kErrWaitEmpty))
+          for (int c = 0; c < n_chunks; ++c, wk += (++wst == p.nst), wst = wst == p.nst ? 0 : wst) {
+            const int st = wst;
+            if ((st & (p.wprod - 1)) != pw) continue;  // with two producers the ring is even
+            if (wk >= 1 && !mbar_wait(bar(w_empty + st), (uint32_t)(wk - 1) & 1u, abort_flag, p.err, kErrWaitEmpty))
               break;
             const int s0 = c * p.sps, s1 = min(p.n_steps, s0 + p.sps);
             if (p.nsplit == 1) {
@@ -348,122 +391,100 @@ __global__ void __launch_bounds__(kThreads, kMaxCtasPerSm) conv_tc_kernel(const 
       if (*abort_flag) break;
     }
   } else if (warp == 1) {
-    // ---------------- MMA issue: one thread ----------------
-    if (lane == 0) {
-      bool ok = !p.resident || mbar_wait(bar(w_full), 0u, abort_flag, p.err, kErrWaitW);
-      const bool fp8 = p.fp8 != 0;
-      const int MT = p.MT, npad = p.ncol;  // accumulator columns of one tile (its slice)
-      const uint32_t idesc = p.idesc;
-      int i = 0;
-      int sa = 0, ka = 0;  // input stage and its use count, advanced without divisions
-      for (int t = blockIdx.x; ok && t < p.n_tiles; t += gridDim.x, ++i, ka += (++sa == na), sa = sa == na ? 0 : sa) {
-        const int s = i & 1, k = i >> 1;     // accumulator buffer
-        const int sl = t & (p.nsplit - 1);   // column slice (nsplit is a power of two)
-        if (!mbar_wait(bar(a_full + sa), (uint32_t)ka & 1u, abort_flag, p.err, kErrWaitA)) break;
-        if (k >= 1 && !mbar_wait(bar(acc_empty + s), (uint32_t)(k - 1) & 1u, abort_flag, p.err, kErrWaitAcc)) break;
-        tc_fence_after();
-        // descriptor start addresses count 16-byte units in their low bits
-        const uint64_t a_stage = (uint64_t)(((uint32_t)sa * (uint32_t)p.a_bytes) >> 4);
-        const uint32_t d0 = tmem + (uint32_t)(s * MT * npad);
-        // the slice's B rows start sl * ncol rows into each K-half (at the
-        // stage's start when the slice is packed)
-        const uint64_t b_slice = p.wcompact ? 0ull : (uint64_t)(sl * p.ncol);
-        for (int c = 0; c < n_chunks; ++c) {
-          uint64_t b_stage = b_slice;
-          int st = 0;
-          if (!p.resident) {
-            const int gc = i * n_chunks + c, use = gc / p.nst;
-            st = gc - use * p.nst;
-            if (!mbar_wait(bar(w_full + st), (uint32_t)use & 1u, abort_flag, p.err, kErrWaitW)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            b_stage = b_slice + (uint64_t)(((uint32_t)st * stage_bytes) >> 4);
+    // ---------------- MMA issue: one elected lane of a converged warp ----------------
+    // every lane walks the same loop (waits included), so that the descriptors
+    // are warp-uniform values (see mma_f16_warp); a wait's verdict is taken
+    // together.  From a single lane's branch the issue bounded every layer with N
+    // below 256: the 2049-tap FIR on 512 rows took 37 us, 26 us so; whitening and
+    // BBHnet on 256 segments 275 -> 260 us (BF16), 235 -> 224 us (FP8).
+    auto wait_all = [&](uint32_t b, uint32_t parity, int code) {
+      return __all_sync(0xffffffffu, mbar_wait(b, parity, abort_flag, p.err, code) ? 1 : 0) != 0;
+    };
+    const uint32_t acc0 = __shfl_sync(0xffffffffu, tmem, 0);
+    bool ok = !p.resident || wait_all(bar(w_full), 0u, kErrWaitW);
+    const bool fp8 = p.fp8 != 0;
+    const int MT = p.MT, npad = p.ncol;  // accumulator columns of one tile (its slice)
+    const uint32_t idesc = p.idesc;
+    int i = 0;
+    int sa = 0, ka = 0;   // input stage and its use count, advanced without divisions
+    int wst = 0, wk = 0;  // the same of the weight ring
+    for (int t = blockIdx.x; ok && t < p.n_tiles; t += gridDim.x, ++i, ka += (++sa == na), sa = sa == na ? 0 : sa) {
+      const int s = i & 1, k = i >> 1;     // accumulator buffer
+      const int sl = t & (p.nsplit - 1);   // column slice (nsplit is a power of two)
+      if (!wait_all(bar(a_full + sa), (uint32_t)ka & 1u, kErrWaitA)) break;
+      if (k >= 1 && !wait_all(bar(acc_empty + s), (uint32_t)(k - 1) & 1u, kErrWaitAcc)) break;
+      tc_fence_after();
+      // descriptor start addresses count 16-byte units in their low bits
+      const uint32_t a_stage = ((uint32_t)sa * (uint32_t)p.a_bytes) >> 4;
+      const uint32_t d0 = acc0 + (uint32_t)(s * MT * npad);
+      // the slice's B rows start sl * ncol rows into each K-half (at the
+      // stage's start when the slice is packed)
+      const uint32_t b_slice = p.wcompact ? 0u : (uint32_t)(sl * p.ncol);
+      for (int c = 0; c < n_chunks; ++c) {
+        uint32_t b_stage = b_slice;
+        const int st = wst;
+        if (!p.resident) {
+          const uint32_t ph = (uint32_t)wk & 1u;
+          wk += (++wst == p.nst);
+          if (wst == p.nst) wst = 0;
+          if (!wait_all(bar(w_full + st), ph, kErrWaitW)) {
+            ok = false;
+            break;
           }
-          const int s0 = p.resident ? 0 : c * p.sps, s1 = p.resident ? p.n_steps : min(p.n_steps, s0 + p.sps);
-          // The issue rate of this one thread bounds the tensor pipe for small
-          // N, so the loop is kept lean: one 16-byte descriptor pair per step,
-          // the next pair loaded while the current MMAs issue.
-          const ulonglong2* tab = reinterpret_cast<const ulonglong2*>(s_desc);
-          if (MT == 1 && p.param_desc) {
-            // descriptors from the parameter table: A start and LBO packed per
-            // step, B at a fixed stride from the stage's first step
-            const uint64_t hi = ((uint64_t)(128u >> 4) << 32) | (1ull << 46);
-            const uint32_t a_base = (sA >> 4) + (uint32_t)a_stage;
-            const uint32_t b_rows = p.wcompact ? (uint32_t)p.ncol : (uint32_t)p.npad;  // K-half distance
-            const uint64_t b_hi = hi | ((uint64_t)((b_rows * 16u) >> 4) << 16);
-            const uint32_t b_base = (sW >> 4) + (uint32_t)b_stage, b_step = (uint32_t)p.wstep >> 4;
-            if (fp8) {
-              for (int sidx = s0; sidx < s1; ++sidx) {
-                const uint32_t e = p.apack[sidx];
-                mma_f8(d0, hi | (uint64_t)((a_base + (e & 0xFFFFu)) & 0x3FFFu) | ((uint64_t)(e >> 16) << 16),
-                       b_hi | (uint64_t)((b_base + (uint32_t)(sidx - s0) * b_step) & 0x3FFFu), idesc,
-                       sidx == 0 ? 0u : 1u);
-              }
-            } else {
-#pragma unroll 4
-              for (int sidx = s0; sidx < s1; ++sidx) {
-                const uint32_t e = p.apack[sidx];
-                mma_f16(d0, hi | (uint64_t)((a_base + (e & 0xFFFFu)) & 0x3FFFu) | ((uint64_t)(e >> 16) << 16),
-                        b_hi | (uint64_t)((b_base + (uint32_t)(sidx - s0) * b_step) & 0x3FFFu), idesc,
-                        sidx == 0 ? 0u : 1u);
-              }
-            }
-            if (!p.resident) mma_commit(bar(w_empty + st));
-            continue;
-          }
-          ulonglong2 cur = tab[s0];
-          if (fp8) {
-            for (int sidx = s0; sidx < s1; ++sidx) {
-              const ulonglong2 nxt = tab[sidx + 1 < s1 ? sidx + 1 : sidx];
-              const uint32_t acc = sidx == 0 ? 0u : 1u;
-              for (int mt = 0; mt < MT; ++mt)  // M sub-tile mt starts 128 rows (2048 bytes) further
-                mma_f8(d0 + (uint32_t)(mt * npad), cur.x + a_stage + (uint64_t)(mt * 128), cur.y + b_stage, idesc,
-                       acc);
-              cur = nxt;
-            }
-          } else if (MT == 1) {
-            // Under load (bulk copies landing, operand reads, epilogue
-            // traffic) a shared-memory read takes longer than issuing several
-            // MMAs, so the descriptor pairs are read four steps ahead.
-            const int last = s1 - 1;
-            ulonglong2 q1 = tab[min(s0 + 1, last)], q2 = tab[min(s0 + 2, last)], q3 = tab[min(s0 + 3, last)];
-            int sidx = s0;
-            for (; sidx + 4 <= s1; sidx += 4) {
-              mma_f16(d0, cur.x + a_stage, cur.y + b_stage, idesc, sidx == 0 ? 0u : 1u);
-              cur = tab[min(sidx + 4, last)];
-              mma_f16(d0, q1.x + a_stage, q1.y + b_stage, idesc, 1u);
-              q1 = tab[min(sidx + 5, last)];
-              mma_f16(d0, q2.x + a_stage, q2.y + b_stage, idesc, 1u);
-              q2 = tab[min(sidx + 6, last)];
-              mma_f16(d0, q3.x + a_stage, q3.y + b_stage, idesc, 1u);
-              q3 = tab[min(sidx + 7, last)];
-            }
-            // fewer than four steps left: they are in cur, q1, q2
-            if (sidx < s1) mma_f16(d0, cur.x + a_stage, cur.y + b_stage, idesc, sidx == 0 ? 0u : 1u);
-            if (sidx + 1 < s1) mma_f16(d0, q1.x + a_stage, q1.y + b_stage, idesc, 1u);
-            if (sidx + 2 < s1) mma_f16(d0, q2.x + a_stage, q2.y + b_stage, idesc, 1u);
-          } else {
-            for (int sidx = s0; sidx < s1; ++sidx) {
-              const ulonglong2 nxt = tab[sidx + 1 < s1 ? sidx + 1 : sidx];
-              const uint32_t acc = sidx == 0 ? 0u : 1u;
-              for (int mt = 0; mt < MT; ++mt)
-                mma_f16(d0 + (uint32_t)(mt * npad), cur.x + a_stage + (uint64_t)(mt * 128), cur.y + b_stage, idesc,
-                        acc);
-              cur = nxt;
-            }
-          }
-          if (!p.resident) mma_commit(bar(w_empty + st));
+          tc_fence_after();
+          b_stage = b_slice + (((uint32_t)st * stage_bytes) >> 4);
         }
-        if (!ok) break;
-        mma_commit(bar(a_empty + sa));
-        mma_commit(bar(acc_full + s));
+        const int s0 = p.resident ? 0 : c * p.sps, s1 = p.resident ? p.n_steps : min(p.n_steps, s0 + p.sps);
+        const uint64_t hi = ((uint64_t)(128u >> 4) << 32) | (1ull << 46);
+        if (MT == 1 && p.param_desc) {
+          // descriptors from the parameter table: A start and LBO packed per
+          // step, B at a fixed stride from the stage's first step
+          const uint32_t a_base = (sA >> 4) + a_stage;
+          const uint32_t b_rows = p.wcompact ? (uint32_t)p.ncol : (uint32_t)p.npad;  // K-half distance
+          const uint64_t b_hi = hi | ((uint64_t)((b_rows * 16u) >> 4) << 16);
+          const uint32_t b_base = (sW >> 4) + b_stage, b_step = (uint32_t)p.wstep >> 4;
+          if (fp8) {
+#pragma unroll 4
+            for (int sidx = s0; sidx < s1; ++sidx) {
+              const uint32_t e = p.apack[sidx];
+              mma_f8_warp(d0, hi | (uint64_t)((a_base + (e & 0xFFFFu)) & 0x3FFFu) | ((uint64_t)(e >> 16) << 16),
+                          b_hi | (uint64_t)((b_base + (uint32_t)(sidx - s0) * b_step) & 0x3FFFu), idesc,
+                          sidx == 0 ? 0u : 1u);
+            }
+          } else {
+#pragma unroll 4
+            for (int sidx = s0; sidx < s1; ++sidx) {
+              const uint32_t e = p.apack[sidx];
+              mma_f16_warp(d0, hi | (uint64_t)((a_base + (e & 0xFFFFu)) & 0x3FFFu) | ((uint64_t)(e >> 16) << 16),
+                           b_hi | (uint64_t)((b_base + (uint32_t)(sidx - s0) * b_step) & 0x3FFFu), idesc,
+                           sidx == 0 ? 0u : 1u);
+            }
+          }
+        } else {
+          // more steps than the parameter table holds, or several M sub-tiles:
+          // descriptors from shared memory, one pair per step
+          const ulonglong2* tab = reinterpret_cast<const ulonglong2*>(s_desc);
+          for (int sidx = s0; sidx < s1; ++sidx) {
+            const ulonglong2 cur = tab[sidx];
+            const uint32_t acc = sidx == 0 ? 0u : 1u;
+            for (int mt = 0; mt < MT; ++mt) {  // M sub-tile mt starts 128 rows (2048 bytes) further
+              const uint64_t ad = cur.x + (uint64_t)(a_stage + (uint32_t)(mt * 128)), bd = cur.y + (uint64_t)b_stage;
+              if (fp8)
+                mma_f8_warp(d0 + (uint32_t)(mt * npad), ad, bd, idesc, acc);
+              else
+                mma_f16_warp(d0 + (uint32_t)(mt * npad), ad, bd, idesc, acc);
+            }
+          }
+        }
+        if (!p.resident) mma_commit_warp(bar(w_empty + st));
       }
-      // all MMAs issued by this thread complete before TMEM is released
-      mma_commit(bar(drain));
-      mbar_wait(bar(drain), 0u, abort_flag, p.err, kErrDrain);
+      if (!ok) break;
+      mma_commit_warp(bar(a_empty + sa));
+      mma_commit_warp(bar(acc_full + s));
     }
+    // all MMAs issued by this warp complete before TMEM is released
+    mma_commit_warp(bar(drain));
+    mbar_wait(bar(drain), 0u, abort_flag, p.err, kErrDrain);
     __syncwarp();
   } else {
     // ---------------- epilogue (warps 2 .. 1 + kEpiWarps): TMEM -> bias/residual/activation -> global ----------------
@@ -1256,6 +1277,10 @@ static void plan_conv_tc(TcParams& q, const LayerDev& L, bool fp8, const TcIn& i
     q.per_sm = per;
   }
   q.n_tiles = q.tiles_per_item * B * q.nsplit;
+  q.nsplit_log = 0;
+  while ((1 << q.nsplit_log) < q.nsplit) ++q.nsplit_log;
+  q.div_tpi = fast_div((uint32_t)q.tiles_per_item);
+  q.prezero = q.tiles_per_item == 1;
   // instruction descriptor: D = F32, A/B = BF16 (kind::f16) or E4M3 (kind::f8f6f4),
   // both K-major, N >> 3 at bit 17, M >> 4 at bit 24 (N = the slice's columns)
   q.idesc = (1u << 4) | (fp8 ? 0u : ((1u << 7) | (1u << 10))) | ((uint32_t)(q.ncol >> 3) << 17) |
