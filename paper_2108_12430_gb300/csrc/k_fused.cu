@@ -221,7 +221,14 @@ struct Smem {
 // buffer (only the producer waits on those, in order).
 enum { kInFull = 0, kInEmpty = kInFull + kSlots, kWFull = kInEmpty + kInBufs, kWEmpty = kWFull + kWStages,
        kAccFull = kWEmpty + kWStages, kActReady = kAccFull + kSlots, kDrain = kActReady + kSlots,
-       kActHalf = kDrain + kSlots, kNBars = kActHalf + kSlots };
+       kActHalf = kDrain + kSlots, kAccFirst = kActHalf + kSlots, kNBars = kAccFirst + kSlots };
+// The barrier that layer l's finished accumulator completes.  The first layer
+// has its own: its MMAs do not wait for the previous item's last epilogue, and
+// that epilogue may be held up by the kernel before this one, so on a common
+// barrier the first layer could complete a second phase before the last
+// layer's was seen, which a parity wait cannot tell from none.  With two
+// barriers the next commit on either one follows the epilogue of the last.
+__device__ constexpr int acc_bar(int l) { return l == 0 ? kAccFirst : kAccFull; }
 
 
 // Descriptor words: low = start address >> 4 (14 bits) | LBO >> 4 << 16, high
@@ -292,7 +299,7 @@ __device__ __forceinline__ bool mma_layer(const Smem& sm, uint32_t tmem, int k, 
   }
   tc_fence_after();
   if (!issue_layer<l>(sm, tmem + acc_col(s, l), k, l == 0 ? sm.input(ib) : sm.act(s), s, act_ph)) return false;
-  mma_commit(sm.bar(kAccFull + s));
+  mma_commit(sm.bar(acc_bar(l) + s));
   if (l == 0) mma_commit(sm.bar(kInEmpty + ib));
   return true;
 }
@@ -336,7 +343,7 @@ __device__ __forceinline__ void epi_hidden(const float (&v)[32], int half, int R
 
 struct EpiItem {
   int rm0[kLayers];
-  int b, t;
+  int b, t, k;  // window, tile, round
 };
 
 // Named barrier 1 + s over the slot's epilogue warps with an AND-reduction:
@@ -358,9 +365,10 @@ __device__ __forceinline__ bool epi_layer(const FParams& p, const Smem& sm, uint
   using F = typename Lay<l>::T;
   const int row = quarter * 32 + lane;  // MMA row = TMEM lane
   bool ok = true;
-  if (poller) ok = mbar_spin(sm.bar(kAccFull + s), (uint32_t)acc_ph & 1u, sm.abort_flag, sm.err, kErrAcc);
+  if (poller)
+    ok = mbar_spin(sm.bar(acc_bar(l) + s), (uint32_t)(l == 0 ? e.k : acc_ph) & 1u, sm.abort_flag, sm.err, kErrAcc);
   if (!epi_bar_and(s, ok)) return false;
-  ++acc_ph;
+  if (l > 0) ++acc_ph;
   tc_fence_after();
   const int R = e.rm0[l] + row;
 #pragma unroll
@@ -423,6 +431,7 @@ __global__ void __launch_bounds__(kThreads, 1) deepclean_fused_kernel(const FPar
     for (int i = 0; i < kSlots; ++i) {
       mbar_init(sm.bar(kInFull + i), 1);
       mbar_init(sm.bar(kAccFull + i), 1);
+      mbar_init(sm.bar(kAccFirst + i), 1);
       mbar_init(sm.bar(kActReady + i), kEpiW);
       mbar_init(sm.bar(kDrain + i), 1);
       mbar_init(sm.bar(kActHalf + i), kEpiW);
@@ -573,6 +582,7 @@ __global__ void __launch_bounds__(kThreads, 1) deepclean_fused_kernel(const FPar
       const int item = (int)blockIdx.x + j * G;
       e.t = item / p.nb;
       e.b = item - e.t * p.nb;
+      e.k = k;
       fused_tile_rows(p.T, p.Lw, e.t, e.rm0, nullptr, nullptr);
       if (!epi_layer<0>(p, sm, tmem, quarter, lane, s, poller, e, acc_ph, s_bias) ||
           !epi_layer<1>(p, sm, tmem, quarter, lane, s, poller, e, acc_ph, s_bias) ||
