@@ -83,41 +83,68 @@ __global__ void serve_push_kernel(const ServeItem* __restrict__ items, ServeGeom
 // Subtraction and aggregation of one new window per item (the window ends at
 // head + S).  AVERAGE: sums per time in window order, divided by the number
 // of windows so far covering the time; LATEST: the newest window alone.
+// Bound: the prediction and the aggregation sums, once each (64 windows of
+// 32768: 25 MB).  A thread takes 4 consecutive samples (W and the rings' lengths
+// are multiples of 4) and only the emitted ones take the 64-bit arithmetic
+// (64 items: 16.0 us one sample at a time, 10.6 us so).
 __global__ void serve_sub_ola_kernel(const ServeItem* __restrict__ items, ServeGeom g, const float* __restrict__ pred) {
   const ServeItem it = items[blockIdx.y];
   if (!it.active) return;
   const int S = it.S, W = g.W;
-  const int64_t head = it.head, k = head / S;
+  const int64_t head = it.head;
   const float* pr = pred + (int64_t)blockIdx.y * W;
   // window sample e is time tau = head + S - W + e; it is emitted as cleaned
   // sample o = e - (W - S - delta) when 0 <= o < S
   const uint32_t R = (uint32_t)g.R, qb = ring_mod(head + S - W, g.R);
-  const uint32_t cb = ring_mod(head - g.delta, g.Rc);
   const int o_shift = W - S - g.delta;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < W; e += gridDim.x * blockDim.x) {
-    const int64_t tau = head + S - W + e;
-    const int o = e - o_shift;
-    const bool emits = o >= 0 && o < S;
-    const uint32_t q = wrap(qb, (uint32_t)e, R);
-    float value;
-    if (g.mode == GW_AGG_LATEST) {
+  const bool vec = (qb & 3u) == 0;
+  for (int e = 4 * (blockIdx.x * blockDim.x + threadIdx.x); e < W; e += 4 * gridDim.x * blockDim.x) {
+    const bool emits = e + 3 >= o_shift && e < o_shift + S;
+    if (g.mode == GW_AGG_LATEST && !emits) continue;
+    const float4 p4 = *reinterpret_cast<const float4*>(pr + e);
+    float v[4] = {p4.x, p4.y, p4.z, p4.w};
+    if (g.mode != GW_AGG_LATEST) {
+      // the sums of times before head; a newer time's slot is an old one's
+      float old[4];
+      float4* a4 = reinterpret_cast<float4*>(it.acc + wrap(qb, (uint32_t)e, R));
+      if (vec) {
+        const float4 q = *a4;
+        old[0] = q.x, old[1] = q.y, old[2] = q.z, old[3] = q.w;
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) old[i] = it.acc[wrap(qb, (uint32_t)(e + i), R)];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = (e + i < W - S ? old[i] : 0.f) + v[i];
+      if (vec) {
+        *a4 = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) it.acc[wrap(qb, (uint32_t)(e + i), R)] = v[i];
+      }
       if (!emits) continue;
-      value = pr[e];
-    } else {
-      const float sum = (tau < head ? it.acc[q] : 0.f) + pr[e];
-      it.acc[q] = sum;
-      if (!emits) continue;
-      const int64_t first = tau >= 0 ? floordiv64(tau, S) : 0;
-      value = sum / (float)(k - first + 1);
     }
-    if (g.post) {
-      // the post-processing FIR reads the aggregated prediction from its ring
-      if (tau >= 0) it.pring[ring_mod(tau, g.Rp)] = value;
-      continue;
+    const int64_t k = head / S;
+    const uint32_t cb = ring_mod(head - g.delta, g.Rc);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int o = e + i - o_shift;
+      if (o < 0 || o >= S) continue;
+      const int64_t tau = head + S - W + e + i;
+      float value = v[i];
+      if (g.mode != GW_AGG_LATEST) {
+        const int64_t first = tau >= 0 ? floordiv64(tau, S) : 0;
+        value /= (float)(k - first + 1);
+      }
+      if (g.post) {
+        // the post-processing FIR reads the aggregated prediction from its ring
+        if (tau >= 0) it.pring[ring_mod(tau, g.Rp)] = value;
+        continue;
+      }
+      const float c = (tau >= 0 ? it.strain[wrap(qb, (uint32_t)(e + i), R)] : 0.f) - value;
+      it.out[o] = c;
+      if (tau >= 0) it.clean[wrap(cb, (uint32_t)o, (uint32_t)g.Rc)] = c;
     }
-    const float c = (tau >= 0 ? it.strain[q] : 0.f) - value;
-    it.out[o] = c;
-    if (tau >= 0) it.clean[wrap(cb, (uint32_t)o, (uint32_t)g.Rc)] = c;
   }
 }
 
@@ -153,52 +180,92 @@ __global__ void serve_post_kernel(const ServeItem* __restrict__ items, ServeGeom
   if (t >= 0) it.clean[ring_mod(t, g.Rc)] = v;
 }
 
-// New decimated samples d[m], m in [m0, m1).
-__global__ void serve_decimate_kernel(const ServeItem* __restrict__ items, ServeGeom g, const float* __restrict__ f,
-                                      int K) {
+// New decimated samples d[m], m in [m0, m1): one per thread, one FMA chain over
+// the taps in order.  A block of taps and the samples that the CTA's outputs
+// take them with are staged in shared memory: the chain's loads were what it
+// waited for (127 taps, 64 items: 8.5 us from the rings, 6.2 us so).
+constexpr int kDecOut = 128, kDecTaps = 512;
+__global__ void __launch_bounds__(kDecOut) serve_decimate_kernel(const ServeItem* __restrict__ items, ServeGeom g,
+                                                                 const float* __restrict__ f, int K) {
+  __shared__ float fs[kDecTaps], xs[2 * kDecOut + kDecTaps];
   const ServeItem it = items[blockIdx.y];
   if (!it.active) return;
   const int c = (K - 1) / 2;
   const uint32_t Rc = (uint32_t)g.Rc;
-  for (int64_t m = it.m0 + blockIdx.x * blockDim.x + threadIdx.x; m < it.m1; m += gridDim.x * blockDim.x) {
-    // taps j with 2m + j - c < 0 read the zeros before the stream start
-    const int64_t jz = c - 2 * m;
-    const int j0 = jz <= 0 ? 0 : (jz > K ? K : (int)jz);
-    uint32_t q = ring_mod(2 * m - c + j0, g.Rc);
+  for (int64_t mb = it.m0 + blockIdx.x * kDecOut; mb < it.m1; mb += gridDim.x * kDecOut) {
+    const int n = (int)min((int64_t)kDecOut, it.m1 - mb);
     float a = 0.f;
-    for (int j = j0; j < K; ++j) {
-      a = fmaf(f[j], it.clean[q], a);
-      q = q + 1 == Rc ? 0u : q + 1;
+    for (int j0 = 0; j0 < K; j0 += kDecTaps) {
+      const int nk = min(kDecTaps, K - j0), nx = 2 * (n - 1) + nk;
+      // the samples before the stream start are zero
+      const int64_t x0 = 2 * mb - c + j0;
+      const uint32_t q0 = ring_mod(x0, g.Rc);
+      for (int i = threadIdx.x; i < nk; i += kDecOut) fs[i] = f[j0 + i];
+      for (int i = threadIdx.x; i < nx; i += kDecOut)
+        xs[i] = x0 + i >= 0 ? it.clean[(q0 + (uint32_t)i) % Rc] : 0.f;
+      __syncthreads();
+      if ((int)threadIdx.x < n)
+        for (int j = 0; j < nk; ++j) a = fmaf(fs[j], xs[2 * threadIdx.x + j], a);
+      __syncthreads();
     }
-    it.dec[ring_mod(m, g.Rd)] = a;
+    if ((int)threadIdx.x < n) it.dec[ring_mod(mb + threadIdx.x, g.Rd)] = a;
   }
 }
 
-// New whitened samples w[n], n in [n0, n1): one CTA per item; the taps and
-// the decimated segment are staged in shared memory, each warp computes one
-// output at a time with its lanes splitting the taps.
-__global__ void serve_whiten_kernel(const ServeItem* __restrict__ items, ServeGeom g, const float* __restrict__ h,
-                                    int K) {
+// New whitened samples w[n], n in [n0, n1): an output's taps go over a warp's
+// lanes (lane j mod 32, each lane's in order, then a tree over the lanes).  The
+// taps and the decimated segment are staged in shared memory.  Bound: the
+// shared-memory loads.  A warp computes kWhitenQ outputs 32 apart, whose samples
+// at one step are the next output's at the step before, in the same lane: a
+// register window takes one new sample and one tap per kWhitenQ FMAs, and an
+// item's outputs go over kWhitenParts CTAs (2049 taps, 64 items of up to 256
+// outputs: 32 us with one output per warp and one CTA per item, 13.7 us so).
+constexpr int kWhitenQ = 8, kWhitenParts = 4;
+__global__ void __launch_bounds__(kThreads) serve_whiten_kernel(const ServeItem* __restrict__ items, ServeGeom g,
+                                                                const float* __restrict__ h, int K) {
   extern __shared__ float sh[];
+  constexpr int Q = kWhitenQ, kWarps = kThreads / 32;
+  static_assert(kWhitenParts * kWarps == 32, "a block of 32 Q outputs: one start per warp");
   const ServeItem it = items[blockIdx.y];
   if (!it.active || it.n1 <= it.n0) return;
   const int c = (K - 1) / 2;
-  const int nn = (int)(it.n1 - it.n0);
+  const int nn = (int)(it.n1 - it.n0), first = blockIdx.x * kWarps;
+  if (first >= nn) return;
   float* hs = sh;
-  float* ds = sh + K;  // d[n0 - c + i], i < nn + K - 1 (< Rd)
+  float* ds = sh + K;  // d[n0 - c + i], i < nn + K - 1 (< Rd), then zeros that only discarded outputs read
   for (int j = threadIdx.x; j < K; j += blockDim.x) hs[j] = h[j];
   const uint32_t Rd = (uint32_t)g.Rd, db = ring_mod(it.n0 - c, g.Rd);
-  for (int i = threadIdx.x; i < nn + K - 1; i += blockDim.x)
-    ds[i] = it.n0 - c + i >= 0 ? it.dec[wrap(db, (uint32_t)i, Rd)] : 0.f;
+  for (int i = threadIdx.x; i < nn + K + 32 * Q; i += blockDim.x)
+    ds[i] = i < nn + K - 1 && it.n0 - c + i >= 0 ? it.dec[wrap(db, (uint32_t)i, Rd)] : 0.f;
   __syncthreads();
   const uint32_t Rw = (uint32_t)g.Rw, wb = ring_mod(it.n0, g.Rw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = warp; i < nn; i += blockDim.x >> 5) {
-    float a = 0.f;
-    for (int j = lane; j < K; j += 32) a = fmaf(hs[j], ds[i + j], a);
+  for (int i = first + warp; i < nn; i += 32 * Q) {
+    const float* x = ds + i + lane;
+    float a[Q], d[Q];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (lane == 0) it.white[wrap(wb, (uint32_t)i, Rw)] = a;
+    for (int q = 0; q < Q; ++q) a[q] = 0.f, d[q] = x[32 * q];
+    int n = 0;
+    for (; 32 * (n + Q) <= K; n += Q) {
+#pragma unroll
+      for (int m = 0; m < Q; ++m) {
+        const float hv = hs[lane + 32 * (n + m)];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) a[q] = fmaf(hv, d[(q + m) % Q], a[q]);
+        d[m] = x[32 * (n + m + Q)];
+      }
+    }
+    for (int j = lane + 32 * n; j < K; j += 32) {
+      const float hv = hs[j];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) a[q] = fmaf(hv, ds[i + j + 32 * q], a[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) a[q] += __shfl_xor_sync(0xffffffffu, a[q], o);
+      if (lane == 0 && i + 32 * q < nn) it.white[wrap(wb, (uint32_t)(i + 32 * q), Rw)] = a[q];
+    }
   }
 }
 
@@ -244,7 +311,7 @@ void launch_serve_push(const ServeItem* items, int n, const ServeGeom& g, int S_
 }
 
 void launch_serve_sub_ola(const ServeItem* items, int n, const ServeGeom& g, const float* pred, cudaStream_t st) {
-  serve_sub_ola_kernel<<<dim3(grid_x(g.W), n), kThreads, 0, st>>>(items, g, pred);
+  serve_sub_ola_kernel<<<dim3(grid_x(g.W / 4), n), kThreads, 0, st>>>(items, g, pred);
   GW_LAUNCH_CHECK();
 }
 
@@ -259,7 +326,7 @@ void launch_serve_post(const ServeItem* items, int n, const ServeGeom& g, const 
 
 void launch_serve_decimate(const ServeItem* items, int n, const ServeGeom& g, const float* taps, int K, int max_new,
                            cudaStream_t st) {
-  serve_decimate_kernel<<<dim3((max_new + 127) / 128, n), 128, 0, st>>>(items, g, taps, K);
+  serve_decimate_kernel<<<dim3((max_new + kDecOut - 1) / kDecOut, n), kDecOut, 0, st>>>(items, g, taps, K);
   GW_LAUNCH_CHECK();
 }
 
@@ -267,10 +334,10 @@ size_t serve_whiten_smem(int K, int max_new) { return (size_t)(2 * K + max_new) 
 
 void launch_serve_whiten(const ServeItem* items, int n, const ServeGeom& g, const float* taps, int K, int max_new,
                          cudaStream_t st) {
-  const size_t smem = serve_whiten_smem(K, max_new);
-  GW_CHECK_ARG(smem <= 200 * 1024, "whitening FIR too long for the streaming kernel");
-  set_smem_limit_once(serve_whiten_kernel, 200 * 1024);
-  serve_whiten_kernel<<<dim3(1, n), kThreads, smem, st>>>(items, g, taps, K);
+  GW_CHECK_ARG(serve_whiten_smem(K, max_new) <= 200 * 1024, "whitening FIR too long for the streaming kernel");
+  const size_t smem = serve_whiten_smem(K, max_new) + 32 * kWhitenQ * sizeof(float);
+  set_smem_limit_once(serve_whiten_kernel, 202 * 1024);
+  serve_whiten_kernel<<<dim3(kWhitenParts, n), kThreads, smem, st>>>(items, g, taps, K);
   GW_LAUNCH_CHECK();
 }
 
