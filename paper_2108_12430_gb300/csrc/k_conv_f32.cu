@@ -186,8 +186,9 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
       }
     }
   };
-  // input standardisation of a landed stage: each thread's own copies
+  // input standardisation of a landed stage, on the rows the warp copied
   auto standardise = [&](int st, int c0) {
+    __syncwarp();
     float* xs = smem + st * t.stage_floats;
     const int n = min(t.CI, s.cin - c0);
     for (int ci = warp; ci < n; ci += nwarps) {
@@ -219,16 +220,14 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
   const int n_chunks = (s.cin + t.CI - 1) / t.CI;
   for (int ch = 0; ch < n_chunks; ++ch) {
     const int st = ch & 1, c0 = ch * t.CI;
+    cp_async_wait<0>();
+    if (a.in_mean) standardise(st, c0);
+    __syncthreads();  // this stage has landed, and every thread is done with the other
     if (ch + 1 < n_chunks) {
       stage_w(st ^ 1, c0 + t.CI);
       stage_x(st ^ 1, c0 + t.CI);
       cp_async_commit();
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
     }
-    if (a.in_mean) standardise(st, c0);
-    __syncthreads();
     const float* xs = smem + st * t.stage_floats;
     const float* ws = xs + t.CI * t.rowp + cg * CPT;
     const int n = min(t.CI, s.cin - c0);
@@ -283,7 +282,6 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
           }
       }
     }
-    __syncthreads();
   }
 
   float v[CPT][PPT];
@@ -299,6 +297,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
   if (t.KS > 1) {
     // partial sums of the other input-channel groups, added in order
     float* red = smem;  // [KS - 1][CPT * PPT][per_k]
+    __syncthreads();    // the last stage has been read
     if (kg > 0) {
 #pragma unroll
       for (int e = 0; e < CPT * PPT; ++e) red[((kg - 1) * CPT * PPT + e) * per_k + r0] = v[e / PPT][e % PPT];
