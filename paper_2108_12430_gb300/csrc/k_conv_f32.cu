@@ -31,9 +31,9 @@
 // first weights while the previous layer ends.
 //
 // Measured (GB300, against scalar FMAs on rows staged through registers, one
-// tile shape): 64 windows of 21 x 32768 in one push 1422 -> 809 us (22 -> 39
+// tile shape): 64 windows of 21 x 32768 in one push 1422 -> 807 us (22 -> 39
 // TFLOP/s; the 32 -> 64 channel layer 304 -> 156 us), whitening and BBHnet on
-// 256 segments 3648 -> 2092 us (its 256 -> 256 layer 947 -> 546 us, 55
+// 256 segments 3648 -> 2007 us (its 256 -> 256 layer 947 -> 546 us, 55
 // TFLOP/s), one window of 21 x 4096 184 -> 40 us.
 #include <algorithm>
 
