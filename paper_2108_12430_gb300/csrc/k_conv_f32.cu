@@ -11,10 +11,15 @@
 // shared-memory loads, operand moves and staging issue beside the FMAs
 // instead of between them.  The pairs are two adjacent output channels: a
 // weight pair is one aligned 64-bit value of shared memory, and an input value
-// is duplicated once per tap for the CPT / 2 pairs it feeds.  Each output
-// is an FP32 FMA chain over (ci, k), input channels in order and taps in order
-// within each, then the bias, so a packed and a scalar chain give the same
-// bits.
+// is duplicated once per tap for the CPT / 2 pairs it feeds.
+//
+// Order of the sums: each output is one FP32 FMA chain over (ci, k), input
+// channels in order and taps in order within each, then the bias, whatever the
+// tile (a packed and a scalar chain give the same bits).  An item's bits
+// therefore do not depend on how many items share its launch: a server's batch
+// follows from arrival times, and a stream's results must not.  So no launch
+// splits the input channels over threads; one with few outputs gives each thread
+// fewer of them instead.
 //
 // Thread: CPT output channels x PPT positions.  Input rows sit in shared
 // memory such that a warp's 16-byte loads walk consecutive addresses: positions
@@ -24,17 +29,15 @@
 //
 // Staging: input channels go through two shared-memory stages of CI channels
 // with their weights, filled by cp.async (zero-filled outside the input: the
-// layer's padding) one chunk ahead of the FMAs.  A CTA's threads can also be
-// split KS ways over the input channels of a chunk; the KS partial sums are
-// added in order at the end.  That split and the small tiles serve launches
+// layer's padding) one chunk ahead of the FMAs.  The small tiles serve launches
 // that would leave the chip idle (plan_conv_f32).  A dependent launch stages its
 // first weights while the previous layer ends.
 //
 // Measured (GB300, against scalar FMAs on rows staged through registers, one
-// tile shape): 64 windows of 21 x 32768 in one push 1422 -> 807 us (22 -> 39
+// tile shape): 64 windows of 21 x 32768 in one push 1422 -> 796 us (22 -> 40
 // TFLOP/s; the 32 -> 64 channel layer 304 -> 156 us), whitening and BBHnet on
-// 256 segments 3648 -> 2007 us (its 256 -> 256 layer 947 -> 546 us, 55
-// TFLOP/s), one window of 21 x 4096 184 -> 40 us.
+// 256 segments 3648 -> 1972 us (its 256 -> 256 layer 947 -> 546 us, 55 TFLOP/s),
+// one window of 21 x 4096 184 -> 41 us.
 #include <algorithm>
 
 #include "gw_internal.h"
@@ -47,7 +50,7 @@ namespace {
 constexpr int kMaxThreads = 256;
 
 struct ConvTile {
-  int CB, np, KS, CI;   // channels, position groups per CTA; input-channel split; channels per stage
+  int CB, np, CI;       // channels, position groups per CTA; input channels per stage
   int lgq;              // log2(CB / 4), or -1 for CB = 1
   int rowp, odd;        // floats per staged input row; offset of its odd samples (stride 2)
   int span;             // samples staged per input row
@@ -138,8 +141,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
   extern __shared__ __align__(16) float smem[];
   const LayerSpec& s = a.s;
   const int tid = threadIdx.x, nthreads = blockDim.x, warp = tid >> 5, lane = tid & 31, nwarps = nthreads >> 5;
-  const int ng = t.CB / CPT, per_k = t.np * ng;
-  const int kg = tid / per_k, r0 = tid - kg * per_k, cg = r0 / t.np, pt = r0 - cg * t.np;
+  const int cg = tid / t.np, pt = tid - cg * t.np;
   const int TL = t.np * PPT;
   const int t0 = blockIdx.x * TL, co0 = blockIdx.y * t.CB, b = blockIdx.z;
   constexpr int XS = (K == 1) ? S : 1;  // input samples per staged sample
@@ -231,7 +233,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
     const float* xs = smem + st * t.stage_floats;
     const float* ws = xs + t.CI * t.rowp + cg * CPT;
     const int n = min(t.CI, s.cin - c0);
-    for (int ci = kg; ci < n; ci += t.KS) {
+    auto channel = [&](int ci) {
       const float* xr = xs + ci * t.rowp + pt * G::XSTEP;
       const float* wr = ws + ci * K * t.CB;
       constexpr int A = G::XSTEP % 4 == 0 ? 4 : 2;
@@ -248,6 +250,8 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
         float w1 = 0.f;
         if constexpr (CPT == 1) {
           w1 = wr[k];
+        } else if constexpr (CPT == 2) {
+          wv[0] = *reinterpret_cast<const f32x2*>(wr + k * t.CB);
         } else {
 #pragma unroll
           for (int q = 0; q < CP / 2; ++q) {
@@ -281,6 +285,14 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
             }
           }
       }
+    };
+    if constexpr (CPT == 8) {
+      for (int ci = 0; ci < n; ++ci) channel(ci);
+    } else {
+      // the next channels' loads run under this one's chain of FMAs (two windows
+      // of 21 x 32768: 69.8 us rolled, 60.1 us so)
+#pragma unroll 4
+      for (int ci = 0; ci < n; ++ci) channel(ci);
     }
   }
 
@@ -293,20 +305,6 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
 #pragma unroll
       for (int c = 0; c < CP; ++c) unpack2(acc[c][j], v[2 * c][j], v[2 * c + 1][j]);
     }
-  }
-  if (t.KS > 1) {
-    // partial sums of the other input-channel groups, added in order
-    float* red = smem;  // [KS - 1][CPT * PPT][per_k]
-    __syncthreads();    // the last stage has been read
-    if (kg > 0) {
-#pragma unroll
-      for (int e = 0; e < CPT * PPT; ++e) red[((kg - 1) * CPT * PPT + e) * per_k + r0] = v[e / PPT][e % PPT];
-    }
-    __syncthreads();
-    if (kg > 0) return;
-    for (int g = 0; g < t.KS - 1; ++g)
-#pragma unroll
-      for (int e = 0; e < CPT * PPT; ++e) v[e / PPT][e % PPT] += red[(g * CPT * PPT + e) * per_k + r0];
   }
 #pragma unroll
   for (int c = 0; c < CPT; ++c) {
@@ -351,13 +349,12 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
 constexpr int kMaxSmem = 110 * 1024;  // two CTAs per SM
 
 template <int K, int S, bool TR2, int CPT, int PPT>
-ConvTile make_tile(const ConvF32Args& a, int CB, int np, int KS) {
+ConvTile make_tile(const ConvF32Args& a, int CB, int np) {
   using G = Geo<K, S, TR2, PPT>;
   const LayerSpec& s = a.s;
   ConvTile t{};
   t.CB = CB;
   t.np = np;
-  t.KS = KS;
   t.cop = conv_f32_cop(s.cout);
   t.flip = s.transposed && s.stride == 1;
   t.pad = t.flip ? K - 1 - s.pad_l : s.pad_l;
@@ -380,7 +377,7 @@ ConvTile make_tile(const ConvF32Args& a, int CB, int np, int KS) {
     t.rowp = ((np * G::NB - 1) * G::BW + (G::NX + 3) / 4 * 4 + 3) / 4 * 4;
   }
   const int per_ci = t.rowp + K * CB;
-  int CI = std::min(s.cin, std::max(KS, 8));
+  int CI = std::min(s.cin, 8);
   while (CI > 1 && (size_t)2 * CI * per_ci * 4 > kMaxSmem) --CI;
   const int chunks = (s.cin + CI - 1) / CI;
   t.CI = (s.cin + chunks - 1) / chunks;
@@ -393,11 +390,11 @@ ConvTile make_tile(const ConvF32Args& a, int CB, int np, int KS) {
 }
 
 template <int K, int S, bool TR2, int CPT, int PPT>
-void launch_tile(const ConvF32Args& a, int CB, int np, int KS, cudaStream_t st) {
-  const ConvTile t = make_tile<K, S, TR2, CPT, PPT>(a, CB, np, KS);
-  const int threads = np * (CB / CPT) * KS;
-  const size_t red = (size_t)(KS - 1) * CPT * PPT * np * (CB / CPT);
-  const size_t smem = std::max<size_t>((size_t)(t.CI < a.s.cin ? 2 : 1) * t.stage_floats, red) * 4;
+void launch_tile(const ConvF32Args& a, int CB, int np, cudaStream_t st) {
+  const ConvTile t = make_tile<K, S, TR2, CPT, PPT>(a, CB, np);
+  const int threads = np * (CB / CPT);
+  GW_CHECK_ARG(threads >= 32 && threads % 32 == 0 && threads <= kMaxThreads, "FP32 conv tile needs whole warps");
+  const size_t smem = (size_t)(t.CI < a.s.cin ? 2 : 1) * t.stage_floats * 4;
   auto kernel = conv_f32_kernel<K, S, TR2, CPT, PPT>;
   set_smem_limit_once(kernel, kMaxSmem);
   cudaLaunchConfig_t cfg{};
@@ -414,19 +411,20 @@ void launch_tile(const ConvF32Args& a, int CB, int np, int KS, cudaStream_t st) 
 }
 
 struct Choice {
-  int cpt, ppt, CB, np, KS;
+  int cpt, ppt, CB, np;
 };
 
 // The tile of a launch.  A thread's tile (channels x positions) sets how many
 // FMAs a loaded value feeds; measured on full launches, 8 x 8 reaches about
 // 0.86 of the FMA rate (256 -> 256 channels, 256 items of 128 positions: 540 us
 // against 560 us for 8 x 4 and 637 us for 4 x 4).  A launch with few outputs
-// does better with smaller tiles, down to 4 x 4 with the input channels split
-// over a CTA's threads: with fewer than about 384 threads per SM the chip idles
-// (32 x 64 x 1024 outputs: 29.6 us at 8 x 8, 26.8 us at 8 x 4; one window of
-// 4096, 64 -> 32 channels: 23.7 us at 8 x 8, 12.3 us at 4 x 4, 7.5 us split 8
-// ways).  The score is that efficiency over the outputs computed, the ones
-// beyond the end of a row included.
+// does better with smaller tiles: with fewer than about 384 threads per SM the
+// chip idles (32 x 64 x 1024 outputs: 29.6 us at 8 x 8, 26.8 us at 8 x 4; one
+// window of 4096, 64 -> 32 channels: 27.2 us at 8 x 8, 18.9 us at 8 x 4, 15.4
+// us at 4 x 4, 13.5 us at 2 x 4; two windows of 32768, the same layer: 16.2 us at
+// 4 x 4, 18.3 us at 2 x 4).  The score is that efficiency over the outputs
+// computed, the ones beyond the end of a row included.  The batch decides only
+// the tile, never the order of a sum.
 Choice plan_conv_f32(const ConvF32Args& a) {
   const LayerSpec& s = a.s;
   const int sms = current_sm_count();
@@ -434,32 +432,31 @@ Choice plan_conv_f32(const ConvF32Args& a) {
   static const struct {
     int cpt, ppt, threads;
     double eff;
-  } kTiles[3] = {{8, 8, 128, 0.86}, {8, 4, 256, 0.80}, {4, 4, 256, 0.70}};
+  } kTiles[4] = {{8, 8, 128, 0.86}, {8, 4, 256, 0.80}, {4, 4, 256, 0.70}, {2, 4, 256, 0.45}};
   int cmax = 8;  // channels per CTA: a power of two, at most 64
   while (cmax < 64 && cmax < s.cout) cmax *= 2;
   Choice best{};
   double best_score = -1;
-  for (int v = 0; v < (one ? 2 : 3); ++v) {
+  for (int v = 0; v < (one ? 2 : 4); ++v) {
     const int ppt = kTiles[v].ppt, cpt = one ? 1 : kTiles[v].cpt;
-    const bool split = v == (one ? 1 : 2);
-    double ks_eff = 1;
-    for (int KS = 1; KS <= (split ? 8 : 1) && KS <= s.cin; KS *= 2, ks_eff *= 0.8) {
-      const int CB = one ? 1 : std::min(cmax, KS == 1 ? 64 : (KS == 2 ? 32 : 16));
-      double np_eff = 1;
-      for (int np = kTiles[v].threads / (CB / cpt) / KS; np >= 8; np /= 2, np_eff *= 0.98) {
-        const int threads = np * (CB / cpt) * KS, TL = np * ppt;
-        if (threads < 64) break;
-        const double tiles = (double)((a.lout + TL - 1) / TL) * ((s.cout + CB - 1) / CB) * a.B;
-        const double useful = (double)a.lout * a.B * s.cout / (tiles * TL * CB);
-        // with 8 channels in all, an 8 x 8 tile leaves too few CTAs per row in
-        // flight (64 x 8 x 32768 outputs: 126 us, 120 us at 8 x 4)
-        const double eff = kTiles[v].eff - (cpt == 8 && ppt == 8 && CB == 8 ? 0.08 : 0.0);
-        const double score =
-            useful * eff * ks_eff * np_eff * std::min(1.0, tiles * threads / (384.0 * sms));
-        if (score > best_score) {
-          best_score = score;
-          best = {cpt, ppt, CB, np, KS};
-        }
+    // 2 x 4: 32 channels per CTA, and 16 of half the threads when even that leaves
+    // two thirds of the SMs without a CTA (BBHnet on one segment 163 us at 64
+    // channels, 143 us at 16; on eight 235 us at 64, 171 us at 32, 222 us at 16)
+    const bool few = cpt == 2 && (double)a.lout * a.B * s.cout * 3 < 256.0 * 8 * sms;
+    const int CB = one ? 1 : std::min(cmax, cpt == 2 ? (few ? 16 : 32) : 64);
+    double np_eff = 1;
+    for (int np = kTiles[v].threads / (few ? 2 : 1) / (CB / cpt); np >= 8; np /= 2, np_eff *= 0.98) {
+      const int threads = np * (CB / cpt), TL = np * ppt;
+      if (threads < 64) break;
+      const double tiles = (double)((a.lout + TL - 1) / TL) * ((s.cout + CB - 1) / CB) * a.B;
+      const double useful = (double)a.lout * a.B * s.cout / (tiles * TL * CB);
+      // with 8 channels in all, an 8 x 8 tile leaves too few CTAs per row in
+      // flight (64 x 8 x 32768 outputs: 126 us, 120 us at 8 x 4)
+      const double eff = kTiles[v].eff - (cpt == 8 && ppt == 8 && CB == 8 ? 0.08 : 0.0);
+      const double score = useful * eff * np_eff * std::min(1.0, tiles * threads / (384.0 * sms));
+      if (score > best_score) {
+        best_score = score;
+        best = {cpt, ppt, CB, np};
       }
     }
   }
@@ -470,20 +467,22 @@ template <int K, int S, bool TR2>
 void launch_shape(const ConvF32Args& a, cudaStream_t st) {
   const Choice c = plan_conv_f32(a);
   if (c.cpt == 8 && c.ppt == 8)
-    launch_tile<K, S, TR2, 8, 8>(a, c.CB, c.np, c.KS, st);
+    launch_tile<K, S, TR2, 8, 8>(a, c.CB, c.np, st);
   else if (c.cpt == 8)
-    launch_tile<K, S, TR2, 8, 4>(a, c.CB, c.np, c.KS, st);
+    launch_tile<K, S, TR2, 8, 4>(a, c.CB, c.np, st);
+  else if (c.cpt == 4)
+    launch_tile<K, S, TR2, 4, 4>(a, c.CB, c.np, st);
   else
-    launch_tile<K, S, TR2, 4, 4>(a, c.CB, c.np, c.KS, st);
+    launch_tile<K, S, TR2, 2, 4>(a, c.CB, c.np, st);
 }
 
 template <int K>
 void launch_one_channel(const ConvF32Args& a, cudaStream_t st) {
   const Choice c = plan_conv_f32(a);
   if (c.ppt == 8)
-    launch_tile<K, 1, false, 1, 8>(a, c.CB, c.np, c.KS, st);
+    launch_tile<K, 1, false, 1, 8>(a, c.CB, c.np, st);
   else
-    launch_tile<K, 1, false, 1, 4>(a, c.CB, c.np, c.KS, st);
+    launch_tile<K, 1, false, 1, 4>(a, c.CB, c.np, st);
 }
 
 }  // namespace
