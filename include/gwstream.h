@@ -509,7 +509,8 @@ int gw_fir_create_band_loss(gw_ctx_t ctx, const double* psd, int n_psd, double f
 int gw_fir_create_bandpass(gw_ctx_t ctx, double fs, int nfft, int ntaps, double f1, double f2, double ramp,
                            int precision, gw_fir_t* out);
 /* loss: device scalar; r: device [B][L - ntaps + 1] (kept for the backward);
- * strain, y_hat: device [B][L]. */
+ * strain, y_hat: device [B][L].  r may lie in the memory of strain or y_hat
+ * (the call then needs room for a second r in the FIR's workspace). */
 int gw_band_loss(gw_fir_t g, const float* strain, const float* y_hat, int B, int L, float* loss, float* r,
                  void* cuda_stream);
 /* dy_hat = dloss * dL/dy_hat = -(2 dloss / N) sum_k g[k] r[m - k]; dloss a

@@ -22,6 +22,8 @@
 // Activation checkpointing: with `checkpoint`, only the inputs of the four
 // blocks (enc1-enc2, enc3-enc4, dec1-dec2, dec3-out) are kept and the first
 // layer's output of each block is recomputed during the backward.
+#include <functional>
+
 #include "gw_train.h"
 
 namespace gw {
@@ -579,7 +581,12 @@ int gw_band_loss(gw_fir_t f, const float* strain, const float* y_hat, int B, int
   GW_CHECK_ARG(f && strain && y_hat && loss && r, "NULL argument");
   GW_CHECK_ARG(B >= 1 && L >= f->ntaps, "need B >= 1 and L >= ntaps");
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  const size_t need = band_loss_part_floats(B, L, f->ntaps) * sizeof(float);
+  // The FIR's CTAs write r while others still read strain and y_hat, so an r in
+  // their memory is made in the workspace and copied at the end.
+  const size_t n_r = (size_t)B * (L - f->ntaps + 1), n_in = (size_t)B * L;
+  auto overlaps = [&](const float* in) { return std::less<const float*>()(r, in + n_in) && std::less<const float*>()(in, r + n_r); };
+  const size_t n_tmp = overlaps(strain) || overlaps(y_hat) ? n_r : 0;
+  const size_t need = (n_tmp + band_loss_part_floats(B, L, f->ntaps)) * sizeof(float);
   if (need > f->ws_bytes) {
     GW_CUDA(cudaStreamSynchronize(st));
     if (f->ws) dev_free(f->ctx, f->ws, f->ws_bytes, nullptr);
@@ -589,7 +596,9 @@ int gw_band_loss(gw_fir_t f, const float* strain, const float* y_hat, int B, int
     f->ws_bytes = need;
   }
   Prof p("band_loss", st);
-  launch_band_loss(strain, y_hat, B, L, f->d_taps, f->ntaps, r, (float*)f->ws, loss, st);
+  float* ws = (float*)f->ws;
+  launch_band_loss(strain, y_hat, B, L, f->d_taps, f->ntaps, n_tmp ? ws : r, ws + n_tmp, loss, st);
+  if (n_tmp) GW_CUDA(cudaMemcpyAsync(r, ws, n_tmp * sizeof(float), cudaMemcpyDeviceToDevice, st));
   GW_API_END
 }
 
