@@ -16,7 +16,7 @@ struct FoldArgs {
   int64_t off_w, off_b, off_g, off_be, off_mu, off_var;
   int cin, cout, K, transposed, bn;
   float* wf;                  // folded [C_in][K][conv_f32_cop(C_out)]
-  float* wT;                  // folded, transposed [C_out][K][conv_f32_cop(C_in)]
+  float* wT;                  // folded, transposed [C_out][K][conv_f32_cop(C_in)], or null
   float* bf;                  // folded bias [C_out]
 };
 
@@ -30,6 +30,7 @@ struct WgradArgs {
   int K, s, p;
   int bias;
   float* partial;
+  size_t partial_cap;  // FP32 kernel: at most this many floats of partials (but at least one CTA's)
 };
 
 // Several layers' folds in one launch (at most kFoldMax).

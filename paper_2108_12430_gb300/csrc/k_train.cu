@@ -49,7 +49,7 @@ __device__ __forceinline__ void fold_body(const FoldArgs& f, int o) {
     const int64_t raw = f.transposed ? ((int64_t)i * f.cout + o) * f.K + k : (int64_t)o * f.cin * f.K + e;
     const float w = (float)((double)f.p[f.off_w + raw] * sc);
     f.wf[((int64_t)i * f.K + k) * conv_f32_cop(f.cout) + o] = w;
-    f.wT[((int64_t)o * f.K + k) * conv_f32_cop(f.cin) + i] = w;
+    if (f.wT) f.wT[((int64_t)o * f.K + k) * conv_f32_cop(f.cin) + i] = w;
   }
 }
 struct FoldList {

@@ -360,7 +360,8 @@ WgTile plan(const WgradArgs& w, int B) {
 
 int parts_of(const WgTile& g, const WgradArgs& w) {
   const int cb_tiles = ((w.NC + 7) / 8 + g.cn - 1) / g.cn;
-  return std::max(1, std::min(g.n_chunks, 2 * current_sm_count() / (g.ab_tiles * cb_tiles)));
+  const int fit = (int)std::min<size_t>(w.partial_cap / g.cols, 1 << 20);
+  return std::max(1, std::min({g.n_chunks, 2 * current_sm_count() / (g.ab_tiles * cb_tiles), fit}));
 }
 
 }  // namespace

@@ -47,7 +47,7 @@ struct TrainLayer {
 // caller): conv, A = the output gradient and Bm = the input; transposed conv,
 // A = the input and Bm = the output gradient; the bias gradient comes with it
 // (bias 1: conv, 2: transposed conv).
-WgradArgs wgrad_plan(const TrainLayer& T) {
+WgradArgs wgrad_plan(const TrainLayer& T, size_t partial_cap) {
   const LayerSpec& s = T.s;
   WgradArgs w{};
   w.NA = s.transposed ? s.cin : s.cout;
@@ -58,6 +58,7 @@ WgradArgs wgrad_plan(const TrainLayer& T) {
   w.s = s.stride;
   w.p = s.pad_l;
   w.bias = s.transposed ? 2 : 1;
+  w.partial_cap = partial_cap;
   return w;
 }
 
@@ -82,7 +83,11 @@ struct gw_trainer {
   std::vector<float*> act;  // output of layer l (l < n_layers - 1), or null when recomputed
   float* scratch = nullptr; // recomputed activation
   float* dv[2] = {nullptr, nullptr};
-  std::vector<float*> partial;  // per layer: the weight gradient's per-CTA partials
+  // the weight gradients' per-CTA partials: layers' one behind the other in one
+  // buffer of partial_floats, added up when the next one's no longer fit
+  float* partial = nullptr;
+  size_t partial_floats = 0, partial_cap = 0;
+  std::vector<size_t> n_partial;  // per layer
   // per layer: the folded parameters' gradients, unfolded after the backward
   std::vector<float*> dWf, dbf;
   float* zero_bias = nullptr;
@@ -221,8 +226,7 @@ int gw_trainer_create(gw_ctx_t ctx, const gw_trainer_desc* d, const float* in_me
     const auto specs = deepclean_specs(d->n_in);
     int64_t off = 0;
     int lin = d->length;
-    size_t max_act = 0;
-    std::vector<size_t> n_partial;
+    size_t max_act = 0;  // a layer's output, per item
     int max_c = 0;
     for (const auto& s : specs) {
       TrainLayer T;
@@ -246,20 +250,36 @@ int gw_trainer_create(gw_ctx_t ctx, const gw_trainer_desc* d, const float* in_me
         f.off_var = off + 3 * s.cout;
         off += 4 * s.cout;
       }
-      max_act = std::max(max_act, (size_t)std::max(s.cin * T.lin, s.cout * T.lout));
+      max_act = std::max(max_act, (size_t)s.cout * T.lout);
       max_c = std::max(max_c, std::max(s.cin, s.cout));
-      const WgradArgs w = wgrad_plan(T);
-      n_partial.push_back(d->precision == GW_BF16 && wgrad_tc_supported(w) ? wgrad_tc_partial_floats(w, d->max_batch)
-                                                                           : wgrad_f32_partial_floats(w, d->max_batch));
       t->layers.push_back(T);
       lin = T.lout;
     }
     GW_CHECK_ARG(lin == d->length, "length does not round-trip through the network");
     t->n_params = (size_t)off;
     const int Bm = d->max_batch;
+    // What the partials may take together: the room that the gradient buffers (and
+    // the recomputed activation) save by not being as large as the network's input,
+    // whose gradient is never computed, and one partial per 256 positions of the
+    // layers with the most weights (32 windows of 21 x 8192: 34.6 MB, and all
+    // layers' partials are 12.3 MB in FP32, 27.9 MB in BF16, so one reduction adds
+    // them all).  One layer's largest partials are the least.
+    const size_t in_act = (size_t)d->n_in * d->length;
+    t->partial_cap = (size_t)Bm * (2 + d->checkpoint) * (in_act > max_act ? in_act - max_act : 0) +
+                     (size_t)Bm * ((d->length + 2047) / 2048) * 64 * 32 * 7;
+    size_t most = 0, all = 0;
+    for (const auto& T : t->layers) {
+      const WgradArgs w = wgrad_plan(T, t->partial_cap);
+      t->n_partial.push_back(t->wgrad_tc && wgrad_tc_supported(w) ? wgrad_tc_partial_floats(w, Bm)
+                                                                  : wgrad_f32_partial_floats(w, Bm));
+      most = std::max(most, t->n_partial.back());
+      all += t->n_partial.back();
+    }
+    t->partial_floats = std::max(most, std::min(all, t->partial_cap));
     for (auto& T : t->layers) {
       T.f.wf = talloc<float>(t, conv_f32_weight_floats(T.s.cin, T.s.cout, T.s.k));
-      T.f.wT = talloc<float>(t, conv_f32_weight_floats(T.s.cout, T.s.cin, T.s.k));
+      // the first layer's input needs no gradient
+      T.f.wT = &T == &t->layers[0] ? nullptr : talloc<float>(t, conv_f32_weight_floats(T.s.cout, T.s.cin, T.s.k));
       T.f.bf = talloc<float>(t, T.s.cout);
     }
     std::vector<float> mean(d->n_in, 0.f), istd(d->n_in, 1.f);
@@ -283,7 +303,7 @@ int gw_trainer_create(gw_ctx_t ctx, const gw_trainer_desc* d, const float* in_me
     if (t->checkpoint) t->scratch = talloc<float>(t, (size_t)Bm * max_act);
     t->dv[0] = talloc<float>(t, (size_t)Bm * max_act);
     t->dv[1] = talloc<float>(t, (size_t)Bm * max_act);
-    for (size_t n : n_partial) t->partial.push_back(talloc<float>(t, n));
+    t->partial = talloc<float>(t, t->partial_floats);
     for (const TrainLayer& T : t->layers) {
       t->dWf.push_back(talloc<float>(t, (size_t)T.s.cin * T.s.cout * T.s.k));
       t->dbf.push_back(talloc<float>(t, T.s.cout));
@@ -446,9 +466,23 @@ int gw_trainer_backward(gw_trainer_t t, const float* dy_hat, float* dparams, voi
   const float* g = dy_hat;  // gradient w.r.t. the current layer's (pre-activation) output
   int64_t gb = t->L, gn = t->L;
   int cur = 0;
-  // weight gradients' partials: added up by one launch at the end
+  // weight gradients' partials, added up when the buffer is full and at the end
   std::vector<WgradReduceItem> reduce;
   std::vector<WgradTcReduceItem> reduce_tc;
+  size_t used = 0;
+  auto add_up = [&] {
+    for (size_t i = 0; i < reduce.size(); i += kWgradReduceMax) {
+      Prof p("train.wgrad_reduce", st);
+      launch_wgrad_reduce(reduce.data() + i, (int)std::min<size_t>(kWgradReduceMax, reduce.size() - i), st);
+    }
+    for (size_t i = 0; i < reduce_tc.size(); i += kWgradReduceMax) {
+      Prof p("train.wgrad_reduce", st);
+      launch_wgrad_tc_reduce(reduce_tc.data() + i, (int)std::min<size_t>(kWgradReduceMax, reduce_tc.size() - i), st);
+    }
+    reduce.clear();
+    reduce_tc.clear();
+    used = 0;
+  };
   TcOut gnext{};  // tc_data: the next data gradient's input, blocked by the previous one
   for (int l = nl - 1; l >= 0; --l) {
     const TrainLayer& T = t->layers[l];
@@ -460,7 +494,7 @@ int gw_trainer_backward(gw_trainer_t t, const float* dy_hat, float* dparams, voi
     }
     const float* xin = layer_input(t, l);
     const int64_t xb = (int64_t)s.cin * T.lin, xc = T.lin;
-    WgradArgs w = wgrad_plan(T);
+    WgradArgs w = wgrad_plan(T, t->partial_cap);
     if (!s.transposed) {
       w.A = g; w.ab = gb; w.aa = gn;
       w.Bm = xin; w.bb = xb; w.bc = xc;
@@ -468,7 +502,9 @@ int gw_trainer_backward(gw_trainer_t t, const float* dy_hat, float* dparams, voi
       w.A = xin; w.ab = xb; w.aa = xc;
       w.Bm = g; w.bb = gb; w.bc = gn;
     }
-    w.partial = t->partial[l];
+    if (used + t->n_partial[l] > t->partial_floats) add_up();
+    w.partial = t->partial + used;
+    used += t->n_partial[l];
     if (t->wgrad_tc && wgrad_tc_supported(w)) {
       Prof p(l < 8 ? kWgradTcNames[l] : "train.wgrad_tc", st);
       reduce_tc.push_back(launch_wgrad_tc(w, B, t->dWf[l], t->dbf[l], t->err, st));
@@ -556,14 +592,7 @@ int gw_trainer_backward(gw_trainer_t t, const float* dy_hat, float* dparams, voi
     gn = xc;
     cur ^= 1;
   }
-  for (size_t i = 0; i < reduce.size(); i += kWgradReduceMax) {
-    Prof p("train.wgrad_reduce", st);
-    launch_wgrad_reduce(reduce.data() + i, (int)std::min<size_t>(kWgradReduceMax, reduce.size() - i), st);
-  }
-  for (size_t i = 0; i < reduce_tc.size(); i += kWgradReduceMax) {
-    Prof p("train.wgrad_reduce", st);
-    launch_wgrad_tc_reduce(reduce_tc.data() + i, (int)std::min<size_t>(kWgradReduceMax, reduce_tc.size() - i), st);
-  }
+  add_up();
   {
     // every layer's chain rule from the folded to the raw parameters, one launch
     std::vector<UnfoldItem> u;
