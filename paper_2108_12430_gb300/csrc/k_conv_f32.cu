@@ -394,6 +394,7 @@ void launch_tile(const ConvF32Args& a, int CB, int np, cudaStream_t st) {
   const ConvTile t = make_tile<K, S, TR2, CPT, PPT>(a, CB, np);
   const int threads = np * (CB / CPT);
   GW_CHECK_ARG(threads >= 32 && threads % 32 == 0 && threads <= kMaxThreads, "FP32 conv tile needs whole warps");
+  GW_CHECK_ARG(t.cop % CB == 0, "FP32 conv tile beyond the padded weight row");
   const size_t smem = (size_t)(t.CI < a.s.cin ? 2 : 1) * t.stage_floats * 4;
   auto kernel = conv_f32_kernel<K, S, TR2, CPT, PPT>;
   set_smem_limit_once(kernel, kMaxSmem);
@@ -433,8 +434,10 @@ Choice plan_conv_f32(const ConvF32Args& a) {
     int cpt, ppt, threads;
     double eff;
   } kTiles[4] = {{8, 8, 128, 0.86}, {8, 4, 256, 0.80}, {4, 4, 256, 0.70}, {2, 4, 256, 0.45}};
-  int cmax = 8;  // channels per CTA: a power of two, at most 64
-  while (cmax < 64 && cmax < s.cout) cmax *= 2;
+  // channels per CTA: a power of two, at most 64, that divides the padded weight
+  // row (a CTA stages its channels of a row unchecked)
+  int cmax = 8;
+  while (cmax < 64 && conv_f32_cop(s.cout) % (2 * cmax) == 0) cmax *= 2;
   Choice best{};
   double best_score = -1;
   for (int v = 0; v < (one ? 2 : 4); ++v) {
