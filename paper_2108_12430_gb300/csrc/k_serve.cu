@@ -84,8 +84,9 @@ __global__ void serve_push_kernel(const ServeItem* __restrict__ items, ServeGeom
 // head + S).  AVERAGE: sums per time in window order, divided by the number
 // of windows so far covering the time; LATEST: the newest window alone.
 // Bound: the prediction and the aggregation sums, once each (64 windows of
-// 32768: 25 MB).  A thread takes 4 consecutive samples (W and the rings' lengths
-// are multiples of 4) and only the emitted ones take the 64-bit arithmetic
+// 32768: 25 MB).  A thread takes 4 consecutive samples (W, every stride and the
+// rings' lengths are multiples of 8, so that they are 16 aligned bytes of the
+// prediction and of the sums) and only the emitted ones take the 64-bit arithmetic
 // (64 items: 16.0 us one sample at a time, 10.6 us so).
 __global__ void serve_sub_ola_kernel(const ServeItem* __restrict__ items, ServeGeom g, const float* __restrict__ pred) {
   const ServeItem it = items[blockIdx.y];
@@ -97,7 +98,6 @@ __global__ void serve_sub_ola_kernel(const ServeItem* __restrict__ items, ServeG
   // sample o = e - (W - S - delta) when 0 <= o < S
   const uint32_t R = (uint32_t)g.R, qb = ring_mod(head + S - W, g.R);
   const int o_shift = W - S - g.delta;
-  const bool vec = (qb & 3u) == 0;
   for (int e = 4 * (blockIdx.x * blockDim.x + threadIdx.x); e < W; e += 4 * gridDim.x * blockDim.x) {
     const bool emits = e + 3 >= o_shift && e < o_shift + S;
     if (g.mode == GW_AGG_LATEST && !emits) continue;
@@ -105,23 +105,12 @@ __global__ void serve_sub_ola_kernel(const ServeItem* __restrict__ items, ServeG
     float v[4] = {p4.x, p4.y, p4.z, p4.w};
     if (g.mode != GW_AGG_LATEST) {
       // the sums of times before head; a newer time's slot is an old one's
-      float old[4];
       float4* a4 = reinterpret_cast<float4*>(it.acc + wrap(qb, (uint32_t)e, R));
-      if (vec) {
-        const float4 q = *a4;
-        old[0] = q.x, old[1] = q.y, old[2] = q.z, old[3] = q.w;
-      } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) old[i] = it.acc[wrap(qb, (uint32_t)(e + i), R)];
-      }
+      const float4 q = *a4;
+      const float old[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i) v[i] = (e + i < W - S ? old[i] : 0.f) + v[i];
-      if (vec) {
-        *a4 = make_float4(v[0], v[1], v[2], v[3]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) it.acc[wrap(qb, (uint32_t)(e + i), R)] = v[i];
-      }
+      *a4 = make_float4(v[0], v[1], v[2], v[3]);
       if (!emits) continue;
     }
     const int64_t k = head / S;
@@ -311,6 +300,7 @@ void launch_serve_push(const ServeItem* items, int n, const ServeGeom& g, int S_
 }
 
 void launch_serve_sub_ola(const ServeItem* items, int n, const ServeGeom& g, const float* pred, cudaStream_t st) {
+  GW_CHECK_ARG(g.W % 8 == 0 && g.R % 8 == 0, "window and ring lengths are multiples of 8");
   serve_sub_ola_kernel<<<dim3(grid_x(g.W / 4), n), kThreads, 0, st>>>(items, g, pred);
   GW_LAUNCH_CHECK();
 }
