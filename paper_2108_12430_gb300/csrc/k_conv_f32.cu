@@ -37,7 +37,7 @@
 // tile shape): 64 windows of 21 x 32768 in one push 1422 -> 796 us (22 -> 40
 // TFLOP/s; the 32 -> 64 channel layer 304 -> 156 us), whitening and BBHnet on
 // 256 segments 3648 -> 1972 us (its 256 -> 256 layer 947 -> 546 us, 55 TFLOP/s),
-// one window of 21 x 4096 184 -> 41 us.
+// one window of 21 x 4096 184 -> 36 us.
 #include <algorithm>
 
 #include "gw_internal.h"
@@ -205,7 +205,11 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
   // the weights do not depend on the previous kernel in the stream
   stage_w(0, 0);
   ptx::griddep_wait();
-  ptx::griddep_launch_dependents();
+  // A launch of small tiles leaves SMs empty; were its dependent let in here, the
+  // next layer's CTAs would crowd on those (BBHnet on eight segments 223 us, 157 us
+  // with the trigger after the FMAs).  A full launch's dependent finds no room
+  // before its end anyway, and the trigger costs nothing here.
+  if (CPT == 8) ptx::griddep_launch_dependents();
   xb = a.item_ptr ? a.item_ptr[b] : a.x + (int64_t)b * a.xb;
   stage_x(0, 0);
   cp_async_commit();
@@ -296,6 +300,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2)
     }
   }
 
+  if (CPT < 8) ptx::griddep_launch_dependents();
   float v[CPT][PPT];
 #pragma unroll
   for (int j = 0; j < PPT; ++j) {
@@ -377,7 +382,12 @@ ConvTile make_tile(const ConvF32Args& a, int CB, int np) {
     t.rowp = ((np * G::NB - 1) * G::BW + (G::NX + 3) / 4 * 4 + 3) / 4 * 4;
   }
   const int per_ci = t.rowp + K * CB;
-  int CI = std::min(s.cin, 8);
+  // Channels per stage: a stage's copies are in flight for the FMAs of one stage.
+  // Eight channels of an 8-channel tile cover that, a small tile's are over before
+  // the copies land (at 8 / 16 / 32 channels: one window of 21 x 4096 40.8 / 38.5 /
+  // 37.2 us, BBHnet on one segment 144 / 130 / 124 us; at eight segments, CTAs of 256
+  // threads, 32 channels take 212 us for 157 at 16).
+  int CI = std::min(s.cin, CPT == 8 ? 8 : (CPT == 2 && np * (CB / CPT) <= 128 ? 32 : 16));
   while (CI > 1 && (size_t)2 * CI * per_ci * 4 > kMaxSmem) --CI;
   const int chunks = (s.cin + CI - 1) / CI;
   t.CI = (s.cin + chunks - 1) / chunks;
@@ -443,8 +453,9 @@ Choice plan_conv_f32(const ConvF32Args& a) {
   for (int v = 0; v < (one ? 2 : 4); ++v) {
     const int ppt = kTiles[v].ppt, cpt = one ? 1 : kTiles[v].cpt;
     // 2 x 4: 32 channels per CTA, and 16 of half the threads when even that leaves
-    // two thirds of the SMs without a CTA (BBHnet on one segment 163 us at 64
-    // channels, 143 us at 16; on eight 235 us at 64, 171 us at 32, 222 us at 16)
+    // two thirds of the SMs without a CTA (BBHnet, at 8 channels per stage: one
+    // segment 163 us at 64 channels, 143 us at 16; eight 235 us at 64, 171 us at 32,
+    // 222 us at 16)
     const bool few = cpt == 2 && (double)a.lout * a.B * s.cout * 3 < 256.0 * 8 * sms;
     const int CB = one ? 1 : std::min(cmax, cpt == 2 ? (few ? 16 : 32) : 64);
     double np_eff = 1;
