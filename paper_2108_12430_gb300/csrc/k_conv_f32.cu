@@ -5,9 +5,9 @@
 // ConvT: y[o,u] = b[o] + sum_{i,k : s | (u + p - k)} w[o,i,k] x[i, (u + p - k) / s]
 // with weights laid out [C_in][K][C_out rounded up to 8] for both.
 //
-// Bound: the FP32 FMA pipe (TF32 could not meet a 1e-5 relative error).  A
-// register-only loop reaches 65 TFLOP/s on the whole chip, scalar and packed
-// alike, but a packed fma.rn.f32x2 does two FMAs per issue slot, so that the
+// Bound: the FP32 FMA pipe (TF32 could not meet a 1e-5 relative error), 80.5
+// TFLOP/s at 2070 MHz.  A register-only loop reaches 76 packed and 75 scalar on
+// the whole chip, but a packed fma.rn.f32x2 does two FMAs per issue slot, so that the
 // shared-memory loads, operand moves and staging issue beside the FMAs
 // instead of between them.  The pairs are two adjacent output channels: a
 // weight pair is one aligned 64-bit value of shared memory, and an input value
@@ -34,9 +34,9 @@
 // first weights while the previous layer ends.
 //
 // Measured (GB300, against scalar FMAs on rows staged through registers, one
-// tile shape): 64 windows of 21 x 32768 in one push 1422 -> 796 us (22 -> 40
+// tile shape): 64 windows of 21 x 32768 in one push 1422 -> 794 us (22 -> 40
 // TFLOP/s; the 32 -> 64 channel layer 304 -> 156 us), whitening and BBHnet on
-// 256 segments 3648 -> 1972 us (its 256 -> 256 layer 947 -> 546 us, 55 TFLOP/s),
+// 256 segments 3648 -> 1971 us (its 256 -> 256 layer 947 -> 546 us, 55 TFLOP/s),
 // one window of 21 x 4096 184 -> 36 us.
 #include <algorithm>
 
@@ -426,16 +426,16 @@ struct Choice {
 };
 
 // The tile of a launch.  A thread's tile (channels x positions) sets how many
-// FMAs a loaded value feeds; measured on full launches, 8 x 8 reaches about
-// 0.86 of the FMA rate (256 -> 256 channels, 256 items of 128 positions: 540 us
-// against 560 us for 8 x 4 and 637 us for 4 x 4).  A launch with few outputs
-// does better with smaller tiles: with fewer than about 384 threads per SM the
-// chip idles (32 x 64 x 1024 outputs: 29.6 us at 8 x 8, 26.8 us at 8 x 4; one
-// window of 4096, 64 -> 32 channels: 27.2 us at 8 x 8, 18.9 us at 8 x 4, 15.4
-// us at 4 x 4, 13.5 us at 2 x 4; two windows of 32768, the same layer: 16.2 us at
-// 4 x 4, 18.3 us at 2 x 4).  The score is that efficiency over the outputs
-// computed, the ones beyond the end of a row included.  The batch decides only
-// the tile, never the order of a sum.
+// FMAs a loaded value feeds; on full launches 256 -> 256 channels, 256 items of
+// 128 positions take 540 us at 8 x 8, 560 us at 8 x 4 and 637 us at 4 x 4, and the
+// tiles' `eff` are about in that ratio (2 x 4: by where it overtakes 4 x 4).  A
+// launch with few outputs does better with smaller tiles: with fewer than about
+// 384 threads per SM the chip idles (32 x 64 x 1024 outputs: 29.6 us at 8 x 8, 26.8
+// us at 8 x 4; one window of 4096, 64 -> 32 channels: 27.2 us at 8 x 8, 18.9 us at
+// 8 x 4, 15.4 us at 4 x 4, 13.5 us at 2 x 4; two windows of 32768, the same layer:
+// 16.2 us at 4 x 4, 18.3 us at 2 x 4; the last two lines at 8 channels per stage).
+// The score is that efficiency over the outputs computed, the ones beyond the end
+// of a row included.  The batch decides only the tile, never the order of a sum.
 Choice plan_conv_f32(const ConvF32Args& a) {
   const LayerSpec& s = a.s;
   const int sms = current_sm_count();

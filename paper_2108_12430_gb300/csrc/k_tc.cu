@@ -877,15 +877,16 @@ int tc_supported() {
 // Output positions folded into one M row (J): enough to make N reach 64
 // columns for small channel counts, bounded so the tap halo stays small.
 //
-// Every tcgen05.mma with M = 128, K = 16 occupies the tensor pipe for the same
-// time whatever its N (up to 256), so the number of (row tile, K-step) pairs
-// sets the cost: folding more positions into N cuts the rows, at the price of
-// more K-steps (the tap halo) and a larger input tile and weight image.
-// Measured on GB300: an M=128, K=16 BF16 MMA costs about 100 cycles at N=64,
-// 112 at N=128 and 143 at N=256 (the last at the dense peak), but layers
-// folded to N=128 ran slower end to end than at N=64 (larger input tiles and
-// weight images, fewer tiles per SM to pipeline).  Target N = 64 and halve J
-// until two input stages plus the resident weights fit in shared memory.
+// A tcgen05.mma with M = 128, K = 16 (BF16) takes the tensor pipe 43 / 50 / 65 /
+// 128 cycles at N = 32 / 64 / 128 / 256: below N = 128 it costs nearly the same
+// whatever its N (reading A is what takes the time), so folding positions into N
+// cuts the rows almost for free, at the price of more K-steps (the tap halo) and a
+// larger input tile and weight image.  N = 128 would halve the rows for a third
+// more per MMA, but layers folded that far ran slower end to end (larger input
+// tiles and weight images, fewer tiles per SM to pipeline); that was measured when
+// one lane issued the MMAs, at about 100 cycles each, and not again since.  Target
+// N = 64 and halve J until two input stages plus the resident weights fit in
+// shared memory.
 static int choose_j(const LayerSpec& s) {
   const int coutp = s.cout == 1 ? 1 : (s.cout + 7) / 8 * 8;
   const int per_j = s.transposed ? 2 * coutp : coutp;

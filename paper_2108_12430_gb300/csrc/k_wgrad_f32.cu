@@ -20,8 +20,8 @@
 // warp tiles, times `tg` groups of runs where the layer has fewer tiles than
 // the CTA warps.  CTAs walk the (item, chunk) list with a grid stride and keep
 // their sums in registers; runs and groups are added in a fixed order, each
-// CTA writes one partial, and one kernel adds every layer's partials in CTA
-// order, so gradients are bitwise reproducible.
+// CTA writes one partial, and one kernel adds the partials of every layer that the
+// trainer's buffer holds in CTA order, so gradients are bitwise reproducible.
 //
 // The bias gradient rides along: conv, the sum of A; transposed conv, the sum
 // of Bm over taps 3 .. 3 + s - 1, which visits every output position once
